@@ -244,6 +244,31 @@ int fft_plan(int n, int *rad_out, std::vector<int> &perm, int needed = 0,
   return (int)rad.size();
 }
 
+// Smallest sphere centred on the axis around the collocation points and
+// interior proxies: the largest distance is convex in the centre.
+void sphere_bounds(const ObsHost &h, ObsDev &d) {
+  auto radius = [](const std::vector<double> &x, int stride, double zc) {
+    double r2 = 0.0;
+    for (size_t i = 0; i + 1 < x.size(); i += stride)
+      r2 = std::max(r2, x[i] * x[i] + (x[i + 1] - zc) * (x[i + 1] - zc));
+    return std::sqrt(r2);
+  };
+  double lo = h.coll[1], hi = h.coll[1];
+  for (size_t i = 0; i < h.coll.size(); i += 4) { lo = std::min(lo, h.coll[i + 1]); hi = std::max(hi, h.coll[i + 1]); }
+  for (size_t i = 0; i < h.src.size(); i += 2) { lo = std::min(lo, h.src[i + 1]); hi = std::max(hi, h.src[i + 1]); }
+  for (int it = 0; it < 60; ++it) {
+    const double a = lo + (hi - lo) / 3.0, b = hi - (hi - lo) / 3.0;
+    const double fa = std::max(radius(h.coll, 4, a), radius(h.src, 2, a));
+    const double fb = std::max(radius(h.coll, 4, b), radius(h.src, 2, b));
+    if (fa < fb) hi = b; else lo = a;
+  }
+  d.sph_zc = 0.5 * (lo + hi);
+  d.sph_rs = radius(h.src, 2, d.sph_zc);
+  d.sph_rt = radius(h.coll, 4, d.sph_zc);
+  d.sph_rho_min = h.coll[0];
+  for (size_t i = 0; i < h.coll.size(); i += 4) d.sph_rho_min = std::min(d.sph_rho_min, h.coll[i]);
+}
+
 axi_status validate(const axi_obstacle &o) {
   if (!o.h_coll || !o.h_src) return AXI_ERR_ARG;
   if (o.bc != AXI_BC_NEUMANN && o.bc != AXI_BC_TRANSMISSION) return AXI_ERR_ARG;
@@ -465,6 +490,7 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
     h.coll.assign(o.h_coll, o.h_coll + 4 * o.M);
     h.src.assign(o.h_src, o.h_src + 2 * o.N);
     if (o.bc == AXI_BC_TRANSMISSION) h.srcx.assign(o.h_src_ext, o.h_src_ext + 2 * o.N);
+    sphere_bounds(h, d);
     h.tab_cos.resize(o.q);
     for (int r = 0; r < o.q; ++r) h.tab_cos[r] = std::cos(2.0 * kPi * r / o.q);
     h.tab_s2.resize(o.q / 2 + 1);

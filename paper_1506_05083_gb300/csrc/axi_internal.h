@@ -124,6 +124,10 @@ struct ObsDev {
   int fft_rad_q[8];
   const int *fft_perm_q;  // [q]
   const double2 *tw_q;    // [q] e^{-2 pi i r / q}
+  // host side only: centre on the axis of the smallest sphere around targets
+  // and interior proxies, the proxies' and targets' radii about it, and the
+  // targets' smallest distance from the axis (near_sph.cu)
+  double sph_zc, sph_rs, sph_rt, sph_rho_min;
 };
 
 __host__ __device__ inline bool owns_mode(const ObsDev &o, int d) {
@@ -304,6 +308,14 @@ size_t near_image_scratch_bytes(const ObsDev &h, int W, double ex, double ey, in
 cudaError_t launch_near_image(const ObsDev *d_o, const ObsDev &h, int W, const double2 *coef,
                               double ex, double ey, const double *dirs, int slices, double2 *U,
                               void *scratch, cudaStream_t st);
+// near_sph.cu: the near-image sum by spherical-wave expansions. Degree of the
+// expansions for a lattice (0: not usable, the direct sum runs), scratch, launch.
+int near_sph_degree(const ObsDev &h, double ex, double ey);
+double near_sph_estimate_us(const ObsDev &h, int W, int p);
+size_t near_sph_scratch_bytes(const ObsDev &h, int W, double ex, double ey, int p);
+cudaError_t launch_near_sph(const ObsDev *d_o, const ObsDev &h, int W, const double2 *coef, double ex,
+                            double ey, const double *dirs, int p, double2 *U, void *scratch,
+                            cudaStream_t st);
 cudaError_t launch_point_strengths(const ObsDev *d_o, const ObsDev &h_o, int W,
                                    const double2 *coef, double2 *sigma, cudaStream_t st);
 

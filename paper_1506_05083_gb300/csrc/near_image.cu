@@ -17,6 +17,10 @@
 // with the image phases. Without the symmetry every image is its own
 // representative with one rotation.
 //
+// Lattices whose images stay clear of the body take near_sph.cu's expansions
+// instead (near_degree below); the rest of this file serves tight lattices,
+// small problems and k D far below 1.
+//
 // Arithmetic: kernel values are generated in FP64 (rsqrt, table sin/cos) and
 // both operands are split into S balanced base-128 digits (ozaki.cuh), written
 // straight into K-major no-swizzle tiles (core matrices of 8 rows x 8 k) of
@@ -439,11 +443,28 @@ int block_targets(const ObsDev &h, int W, int nrot) {
   return rings * h.P;
 }
 
+// Degree of the spherical-wave expansions (near_sph.cu) that replace a split
+// sum, 0 for the direct sum below. They run where the lattice allows them and
+// the direct sum would take longer: about 80 us of launches and 0.145 ns a
+// kernel value per representative image (both measured, the same for 1 to 64
+// waves). On a 24-ring body in a tight lattice (p = 105, 5 waves) the two meet:
+// 230 us direct with two representatives, 770 with eight, 400 by expansions.
+// The direct FP64 sum (slices 0) stays what it says.
+int near_degree(const ObsDev &h, const NearGeom &g, int slices) {
+  if (slices <= 0) return 0;
+  const int p = near_sph_degree(h, g.ex, g.ey);
+  if (p == 0) return 0;
+  const double direct = g.nrep * (80.0 + 1.45e-4 * g.S * ((double)h.M * h.P));
+  return near_sph_estimate_us(h, g.W, p) < direct ? p : 0;
+}
+
 }  // namespace
 
 size_t near_image_scratch_bytes(const ObsDev &h, int W, double ex, double ey, int slices) {
   const NearGeom g = make_geom(h, W, ex, ey);
   const size_t T = (size_t)h.M * h.P;
+  const int p = near_degree(h, g, slices);
+  if (p > 0) return near_sph_scratch_bytes(h, W, ex, ey, p);
   size_t b = 0;
   auto add = [&](size_t n) { b += (n + 255) & ~(size_t)255; };
   add(sizeof(double2) * (size_t)W * h.cols * h.P);     // sigma
@@ -510,6 +531,8 @@ cudaError_t launch_near_image(const ObsDev *d_o, const ObsDev &h, int W, const d
                               double ex, double ey, const double *dirs, int slices, double2 *U,
                               void *scratch, cudaStream_t st) {
   const int T = h.M * h.P;
+  const int p = near_degree(h, make_geom(h, W, ex, ey), slices);
+  if (p > 0) return launch_near_sph(d_o, h, W, coef, ex, ey, dirs, p, U, scratch, st);
   char *sc = static_cast<char *>(scratch);
   double2 *sigma = reinterpret_cast<double2 *>(sc);
   sc += (sizeof(double2) * (size_t)W * h.cols * h.P + 255) & ~(size_t)255;
