@@ -30,7 +30,7 @@ struct ObsHost {
   size_t off_coll, off_src, off_srcx, off_cos, off_s2, off_tw, off_A, off_tau, off_T;
   size_t off_ring = 0;
   std::vector<double2> tab_ring;
-  size_t off_svdU = 0, off_svdV = 0, off_svdS = 0, off_svdSw = 0;
+  size_t off_svdU = 0, off_svdV = 0, off_svdS = 0, off_svdSw = 0, off_svdPerm = 0;
   size_t off_ybuf = 0, off_ykey = 0, off_ydig = 0, off_yexp = 0;
   size_t off_vdig = 0, off_vexp = 0, off_ckey = 0, off_rdig = 0, off_rex = 0, off_perm = 0, off_perm_q = 0, off_tw_q = 0;
   std::vector<unsigned short> fill_cdig;   // split fill: cos-table digits [S][2 MR][Lp]
@@ -536,6 +536,7 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
       h.off_svdV = off; off = align_up(off + sizeof(double2) * (size_t)d.D * d.cols * d.cols);
       h.off_svdS = off; off = align_up(off + sizeof(double) * (size_t)d.D * d.cols);
       h.off_svdSw = off; off = align_up(off + sizeof(int) * (size_t)d.D);
+      h.off_svdPerm = off; off = align_up(off + sizeof(int) * (size_t)d.D * d.cols);
     }
     if (slices > 0) {
       // digit rows: rounded up to 64, plus 64 zero rows so that a 64-row chunk
@@ -831,6 +832,7 @@ axi_status axi_build_operator(axi_plan *plan, void *d_workspace, size_t bytes, v
     d.svdV = d.tsvd ? reinterpret_cast<double2 *>(ws + h.off_svdV) : nullptr;
     d.svdS = d.tsvd ? reinterpret_cast<double *>(ws + h.off_svdS) : nullptr;
     d.svdSweeps = d.tsvd ? reinterpret_cast<int *>(ws + h.off_svdSw) : nullptr;
+    d.svdPerm = d.tsvd ? reinterpret_cast<int *>(ws + h.off_svdPerm) : nullptr;
     d.vdig = d.slices > 0 ? reinterpret_cast<unsigned short *>(ws + h.off_vdig) : nullptr;
     d.vexp = d.slices > 0 ? reinterpret_cast<int *>(ws + h.off_vexp) : nullptr;
     d.ckey = d.slices > 0 ? reinterpret_cast<unsigned long long *>(ws + h.off_ckey) : nullptr;

@@ -116,6 +116,7 @@ struct ObsDev {
   double2 *svdU, *svdV;   // [D][cols][cols] column-major
   double *svdS;           // [D][cols]
   int *svdSweeps;         // [D] Jacobi sweeps taken
+  int *svdPerm;           // [D][cols] pivots of the preconditioning QR
   int fft_nst;            // radices of P for the apply's FFTs (0: P has other prime factors)
   int fft_rad[8];
   const int *fft_perm;    // [P] position of output n after the in-place FFT
@@ -221,6 +222,25 @@ bool q_shape(const axi_cell &c, long long &rows, long long &cols, long long &nrb
 bool q_modes(const axi_cell &c, int *mn, long long cap);
 cudaError_t launch_q(const ObsDev *d_obs, const ObsDev &h, int oi, const axi_cell &c, double2 *out,
                      long long ld, cudaStream_t st);
+// Jacobi SVDs (svd_dense.cu) of matrices A [m x n] (strides lda, sA), m >= n: on
+// return A = U (or U Sigma), V [n x n], S = sigma [n]. state: per matrix, the
+// sweeps and flags below (batches only).
+struct SvdBatch {
+  double2 *A;
+  long long lda, sA;
+  double2 *V;
+  long long ldv, sV;
+  double *S;
+  long long sS;
+  int *state;
+  const unsigned char *owned;   // [nmat] matrices to work on, or null
+  int m, n;
+};
+constexpr int kSvdRotated = 1 << 30, kSvdDone = 1 << 29;
+// Batch of nmat matrices, asynchronous; perm: [nmat][n] scratch; U unscaled.
+bool svd_batch_fits(int n, int m);
+cudaError_t svd_batch(const SvdBatch &q, int nmat, int *perm, double tol, int max_sweeps, int *status,
+                      cudaStream_t st);
 // Dense SVD for Q^+ (svd_dense.cu): one-sided Jacobi (A <- U Sigma, V, sigma;
 // *converged false when max_sweeps ran out) and the truncated solve.
 cudaError_t svd_jacobi(double2 *A, long long m, long long n, long long lda, double2 *V, long long ldv,

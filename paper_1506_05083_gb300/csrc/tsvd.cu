@@ -6,6 +6,9 @@
 //   c = V Sigma^+ U_R^H (Q^H fhat_n)_{1:N},
 // Sigma^+ keeping the singular values >= 1e-10 sigma_max.
 //
+// R's SVD is the batched block Jacobi of svd_dense.cu. Blocks too wide for its
+// shared memory (n above 3400) take the kernel below, one CTA per mode.
+//
 // One-sided (Hestenes) Jacobi: the columns g_i of G (initially R) are made
 // mutually orthogonal by plane rotations from the right, G <- G J, V <- V J.
 // For a pair (i, j) with alpha = |g_i|^2, beta = |g_j|^2, gamma = g_i^H g_j,
@@ -36,6 +39,18 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // Column k of round r of the circle method over m (even) positions.
 __device__ __forceinline__ int circle_pos(int k, int r, int m) {
   return k == 0 ? 0 : 1 + (k - 1 + r) % (m - 1);
+}
+
+// R, zeros below the diagonal, into U's storage.
+__global__ void __launch_bounds__(256)
+tsvd_copy_r_kernel(const ObsDev *__restrict__ od) {
+  const ObsDev &o = *od;
+  const int d = blockIdx.y, n = o.cols;
+  const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (e >= (long long)n * n || !owns_mode(o, d)) return;
+  const int j = (int)(e / n), i = (int)(e % n);
+  o.svdU[(size_t)d * n * n + e] =
+      i <= j ? o.A[(size_t)d * n * o.rows + (size_t)j * o.rows + i] : make_double2(0.0, 0.0);
 }
 
 __global__ void __launch_bounds__(kJThreads)
@@ -222,6 +237,12 @@ tsvd_apply_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int nc
 }  // namespace
 
 cudaError_t launch_tsvd(const ObsDev *d_o, const ObsDev &h, cudaStream_t st) {
+  if (svd_batch_fits(h.cols, h.cols)) {
+    const long long n = h.cols;
+    tsvd_copy_r_kernel<<<dim3((unsigned)((n * n + 255) / 256), h.D), 256, 0, st>>>(d_o);
+    const SvdBatch q{h.svdU, n, n * n, h.svdV, n, n * n, h.svdS, n, h.svdSweeps, h.mode_owned, h.cols, h.cols};
+    return svd_batch(q, h.D, h.svdPerm, h.cols * kEps, kMaxSweeps, h.status, st);
+  }
   const size_t smem = (sizeof(double) + sizeof(int)) * (size_t)h.cols + 16;
   static size_t granted = 0;
   cudaError_t e = ensure_dynamic_smem(tsvd_jacobi_kernel, smem, granted);
