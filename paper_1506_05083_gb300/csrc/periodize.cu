@@ -49,6 +49,7 @@
 
 #include "axi_internal.h"
 #include "fft.cuh"
+#include "trig.cuh"
 
 namespace axi {
 namespace {
@@ -441,13 +442,33 @@ q_w_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__re
 //   u_F - beta u_B  = sum_a alpha^a (beta^-1 Psi(x_B - a e_x + 2 e_y)
 //                                    - beta^2 Psi(x_B - a e_x - e_y)),
 // and the same for the derivative rows; T and D keep all nine images. One
-// warp per (row pair, ring j): per image point the lanes form the P samples
-// of G and of one Cartesian derivative of G, two warp FFTs give every mode,
-// and the image's coefficient times both is added in shared memory; the
-// row pair's two rows are written for all P modes (column (n mod P) N + j).
+// warp per (row pair, ring j): the lanes form the P samples of G and of one
+// Cartesian derivative of G, each summed over the images with their
+// coefficients (the same for every sample, so the sum and the transform
+// exchange), and two warp FFTs give every mode; the row pair's two rows are
+// written for all P modes (column (n mod P) N + j). The FP64 pipe bounds it: 33
+// operations a sample and image (sin and cos in fixed point, table through
+// L1), and one pair of FFTs a row pair instead of one an image. 2048 x 15570
+// entries, P = 90: 32.6 ms with an FFT pair an image and the library's sincos,
+// now 10.8 ms.
 // ---------------------------------------------------------------------------
 
 constexpr int kCWarps = 4;
+
+__device__ const long long g_c_ring_q62[trig::kRingTab][2] = {
+#include "ring_table_q62.inc"
+};
+
+__device__ __forceinline__ void c_sincos(double x, double *sn, double *cs) {
+  if (fabs(x) < 1048576.0)
+    trig::sincos_ring_q(x, reinterpret_cast<const longlong2 *>(g_c_ring_q62), sn, cs);
+  else
+    sincos(x, sn, cs);
+}
+
+// Shared memory of c_kernel: twiddles, FFT positions, and per warp the samples
+// of both rows and nine images of (x, y, coefficient).
+__host__ __device__ inline size_t c_warp_smem(int P) { return 2 * (size_t)P + 18; }   // in double2
 
 __global__ void __launch_bounds__(32 * kCWarps)
 c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__restrict__ out, long long ld) {
@@ -457,8 +478,8 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
   extern __shared__ double2 c_sh[];
   double2 *tw = c_sh;                                           // [P] e^{-2 pi i r / P}
   int *perm = reinterpret_cast<int *>(c_sh + P);                // [P]
-  double2 *ws = c_sh + P + (P + 1) / 2 + (size_t)warp * 4 * P;  // value, derivative, their sums
-  double2 *sv = ws, *sd = ws + P, *av = ws + 2 * P, *ad = ws + 3 * P;
+  double2 *sv = c_sh + P + (P + 1) / 2 + (size_t)warp * c_warp_smem(P), *sd = sv + P;
+  double2 *img = sd + P;                                        // [9][2]: point (x, y), coefficient
   const bool fft = o.fft_nst > 0;
   for (int i = threadIdx.x; i < P; i += blockDim.x) {
     tw[i] = o.tw_P[i];
@@ -474,20 +495,17 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
   const double ex = cell.ex, ey = cell.ey, hx = 0.5 * ex, hy = 0.5 * ey, z0 = cell.z0;
   const double k = o.k, rs = o.src[2 * j], zs = o.src[2 * j + 1];
   const double wgt = 1.0 / (4.0 * 3.14159265358979323846 * P);
-  double2 al, be;
-  sincos(cell.kx * ex, &al.y, &al.x);
-  sincos(cell.ky * ey, &be.y, &be.x);
-  const double2 al_inv = make_double2(al.x, -al.y), be_inv = make_double2(be.x, -be.y);
-  const double2 al2 = cmul2(al, al), be2 = cmul2(be, be);
-  for (int n = lane; n < P; n += 32) {
-    av[n] = make_double2(0.0, 0.0);
-    ad[n] = make_double2(0.0, 0.0);
-  }
   const int axis = grp == 0 ? 0 : grp == 1 ? 1 : 2;
   const int npts = grp < 2 ? 6 : 9;
-  bool finite = true;
-  for (int t = 0; t < npts; ++t) {
-    double x, y, z;
+  const double z = grp == 2 ? z0 : grp == 3 ? -z0 : z0 * gb, dz = z - zs, dz2 = dz * dz;
+  if (lane < npts) {                                            // lane t: image t
+    const int t = lane;
+    double2 al, be;
+    sincos(cell.kx * ex, &al.y, &al.x);
+    sincos(cell.ky * ey, &be.y, &be.x);
+    const double2 al_inv = make_double2(al.x, -al.y), be_inv = make_double2(be.x, -be.y);
+    const double2 al2 = cmul2(al, al), be2 = cmul2(be, be);
+    double x, y;
     double2 cf;
     if (grp == 0) {                                  // b = t % 3 - 1; far right / far left images
       const int b = t % 3 - 1;
@@ -495,7 +513,6 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
       const bool right = t < 3;
       x = right ? -hx + 2.0 * ex : -hx - ex;
       y = hy * ga - b * ey;
-      z = z0 * gb;
       cf = right ? cmul2(al_inv, bb) : cmul2(make_double2(-al2.x, -al2.y), bb);
     } else if (grp == 1) {
       const int a = t % 3 - 1;
@@ -503,7 +520,6 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
       const bool front = t < 3;
       x = hx * ga - a * ex;
       y = front ? -hy + 2.0 * ey : -hy - ey;
-      z = z0 * gb;
       cf = front ? cmul2(aa, be_inv) : cmul2(aa, make_double2(-be2.x, -be2.y));
     } else {
       const int a = t / 3 - 1, b = t % 3 - 1;
@@ -511,55 +527,64 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
       const double2 bb = b < 0 ? be_inv : b > 0 ? be : make_double2(1.0, 0.0);
       x = hx * ga - a * ex;
       y = hy * gb - b * ey;
-      z = grp == 2 ? z0 : -z0;
       cf = cmul2(aa, bb);
     }
-    for (int sidx = lane; sidx < P; sidx += 32) {
-      // y_j(psi_s) = (rs cos psi_s, rs sin psi_s, zs); cos, sin from the twiddle table
-      const double dx = x - rs * tw[sidx].x, dy = y + rs * tw[sidx].y, dz = z - zs;
-      const double R2 = dx * dx + dy * dy + dz * dz;
-      const double iR = rsqrt(R2), R = R2 * iR, kR = k * R;
-      double sn, cs;
-      sincos(kR, &sn, &cs);
-      const double g = wgt * iR;
-      sv[sidx] = make_double2(cs * g, sn * g);
-      const double dc = axis == 0 ? dx : axis == 1 ? dy : dz;
-      const double f = dc * g * iR * iR;               // (x - y)_c (ikR - 1) e^{ikR} / (4 pi P R^3)
-      sd[sidx] = make_double2(f * fma(-kR, sn, -cs), f * fma(kR, cs, -sn));
-    }
-    __syncwarp();
-    if (fft) {
-      fft::warp_fft(sv, P, tw, o.fft_rad, o.fft_nst, lane);
-      fft::warp_fft(sd, P, tw, o.fft_rad, o.fft_nst, lane);
-      // sum_s a_s e^{+2 pi i n s / P} is the forward transform at -n mod P
-      for (int n = lane; n < P; n += 32) {
-        const int pos = perm[(P - n) % P];
-        const double2 v = cmul2(cf, sv[pos]), d = cmul2(cf, sd[pos]);
-        av[n] = make_double2(av[n].x + v.x, av[n].y + v.y);
-        ad[n] = make_double2(ad[n].x + d.x, ad[n].y + d.y);
-      }
-    } else {                                          // direct sums for P with other prime factors
-      for (int n = lane; n < P; n += 32) {
-        double2 v = make_double2(0.0, 0.0), d = make_double2(0.0, 0.0);
-        for (int sidx = 0; sidx < P; ++sidx) {
-          const double2 e = make_double2(tw[((long long)n * sidx) % P].x, -tw[((long long)n * sidx) % P].y);
-          v = make_double2(v.x + sv[sidx].x * e.x - sv[sidx].y * e.y, v.y + sv[sidx].x * e.y + sv[sidx].y * e.x);
-          d = make_double2(d.x + sd[sidx].x * e.x - sd[sidx].y * e.y, d.y + sd[sidx].x * e.y + sd[sidx].y * e.x);
-        }
-        v = cmul2(cf, v);
-        d = cmul2(cf, d);
-        av[n] = make_double2(av[n].x + v.x, av[n].y + v.y);
-        ad[n] = make_double2(ad[n].x + d.x, ad[n].y + d.y);
-      }
-    }
-    __syncwarp();
+    img[2 * t] = make_double2(x, y);
+    img[2 * t + 1] = make_double2(wgt * cf.x, wgt * cf.y);
   }
+  __syncwarp();
+  bool finite = true;
+  for (int sidx = lane; sidx < P; sidx += 32) {
+    // y_j(psi_s) = (rs cos psi_s, rs sin psi_s, zs); cos, sin from the twiddle table
+    const double yx = rs * tw[sidx].x, yy = -rs * tw[sidx].y;
+    double2 v = make_double2(0.0, 0.0), d = v;
+    for (int t = 0; t < npts; ++t) {
+      const double2 pt = img[2 * t], cf = img[2 * t + 1];
+      const double dx = pt.x - yx, dy = pt.y - yy;
+      const double R2 = fma(dx, dx, fma(dy, dy, dz2));
+      const double iR = rsqrt(R2), kR = k * (R2 * iR);
+      double sn, cs;
+      c_sincos(kR, &sn, &cs);
+      const double gr = cs * iR, gi = sn * iR;
+      const double dc = axis == 0 ? dx : axis == 1 ? dy : dz;
+      const double f = dc * (iR * iR);                 // (x - y)_c (ikR - 1) e^{ikR} / (4 pi P R^3)
+      const double hr = f * fma(-kR, gi, -gr), hi = f * fma(kR, gr, -gi);
+      v.x = fma(cf.x, gr, fma(-cf.y, gi, v.x));
+      v.y = fma(cf.x, gi, fma(cf.y, gr, v.y));
+      d.x = fma(cf.x, hr, fma(-cf.y, hi, d.x));
+      d.y = fma(cf.x, hi, fma(cf.y, hr, d.y));
+    }
+    sv[sidx] = v;
+    sd[sidx] = d;
+  }
+  __syncwarp();
   const long long r0 = (long long)(2 * grp) * nr + idx, r1 = r0 + nr;
+  if (fft) {
+    fft::warp_fft(sv, P, tw, o.fft_rad, o.fft_nst, lane);
+    fft::warp_fft(sd, P, tw, o.fft_rad, o.fft_nst, lane);
+  }
   for (int n = lane; n < P; n += 32) {
+    double2 v, d;
+    if (fft) {
+      // sum_s a_s e^{+2 pi i n s / P} is the forward transform at -n mod P
+      const int pos = perm[(P - n) % P];
+      v = sv[pos];
+      d = sd[pos];
+    } else {                                            // direct sums for P with other prime factors
+      v = d = make_double2(0.0, 0.0);
+      int t = 0;                                        // n s mod P
+      for (int sidx = 0; sidx < P; ++sidx) {
+        const double2 e = make_double2(tw[t].x, -tw[t].y);
+        v = make_double2(v.x + sv[sidx].x * e.x - sv[sidx].y * e.y, v.y + sv[sidx].x * e.y + sv[sidx].y * e.x);
+        d = make_double2(d.x + sd[sidx].x * e.x - sd[sidx].y * e.y, d.y + sd[sidx].x * e.y + sd[sidx].y * e.x);
+        t += n;
+        if (t >= P) t -= P;
+      }
+    }
     const long long col = (long long)n * N + j;
-    out[col * ld + r0] = av[n];
-    out[col * ld + r1] = ad[n];
-    finite = finite && isfinite(av[n].x + av[n].y + ad[n].x + ad[n].y);
+    out[col * ld + r0] = v;
+    out[col * ld + r1] = d;
+    finite = finite && isfinite(v.x + v.y + d.x + d.y);
   }
   if (!__all_sync(0xffffffffu, finite) && lane == 0) atomicOr(o.status, kStatNonFinite);
 }
@@ -695,7 +720,7 @@ cudaError_t launch_c(const ObsDev *d_obs, const ObsDev &h, int oi, const axi_cel
   static thread_local QCell q;
   if (!make_qcell(c, q)) return cudaErrorInvalidValue;
   const int P = h.P;
-  const size_t smem = sizeof(double2) * ((size_t)P + (P + 1) / 2 + (size_t)kCWarps * 4 * P);
+  const size_t smem = sizeof(double2) * ((size_t)P + (P + 1) / 2 + kCWarps * c_warp_smem(P));
   static size_t granted = 0;
   cudaError_t e = ensure_dynamic_smem(c_kernel, smem, granted);
   if (e != cudaSuccess) return e;
