@@ -739,7 +739,8 @@ static axi_status run_build(axi_operator_s *op, cudaStream_t st,
               ? axi::launch_qr_update_next_split(op->d_obs, op->d_task_obs, op->d_task_mode, nt,
                                                  (int)s, slices, p->step_rows[s],
                                                  p->tune.next_cluster, st)
-              : axi::launch_qr_update_next(op->d_obs, op->d_task_obs, op->d_task_mode, nt, (int)s, st);
+              : axi::launch_qr_update_next(op->d_obs, op->d_task_obs, op->d_task_mode, nt, (int)s, p->step_rows[s],
+                                           st);
       axi::prof_end(pid, st, p->step_fl_next[s]);
       if (e != cudaSuccess) return AXI_ERR_CUDA;
     }

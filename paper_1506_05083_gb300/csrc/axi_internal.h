@@ -187,7 +187,8 @@ inline void prefer_max_shared(Kernel *kernel) {
 // attribute calls.
 template <typename Kernel>
 inline cudaError_t ensure_dynamic_smem(Kernel *kernel, size_t bytes, size_t &granted) {
-  if (bytes <= 48 * 1024 || bytes <= granted) return cudaSuccess;
+  // the default limit of 48 KB counts static shared memory too (at most 16 KB here)
+  if (bytes <= 32 * 1024 || bytes <= granted) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess) granted = bytes;
   return e;
@@ -262,7 +263,7 @@ cudaError_t launch_qr_panel_fx(const ObsDev *d_obs, const int *d_task_obs, const
 // Trailing update of panel step `panel`: the next panel's kNB columns (native
 // FP64, critical path), and the columns beyond (split or FP64; col_off = kNB).
 cudaError_t launch_qr_update_next(const ObsDev *d_obs, const int *d_task_obs,
-                                  const int *d_task_mode, int ntasks, int panel, cudaStream_t st);
+                                  const int *d_task_mode, int ntasks, int panel, int max_rows, cudaStream_t st);
 // Split plans: digits of panel p's reflectors over the whole GPU, after a
 // panel kernel that wrote the reflector columns' exponents.
 cudaError_t launch_vdigits(const ObsDev *d_obs, const int *d_task_obs, const int *d_task_mode,

@@ -598,36 +598,137 @@ qr_update_kernel(const ObsDev *__restrict__ obs, const int *__restrict__ task_ob
                               ncols, sm);
 }
 
-// Q^H applied to the RHS block of mode d: X_d is [2W][rows] column-major.
-// Narrow tiles (kTA columns, 128 threads) give several CTAs per mode: the 12+
-// panel applications of one tile are sequential, so parallelism comes from
-// modes x tiles.
-constexpr int kTA = 8;
-__global__ void __launch_bounds__(kNB * kTA)
-apply_qh_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int ncols_total) {
+// The same with the rows dealt out over a cluster of C = 1, 2, 4 or 8 CTAs in
+// turns of 8: row i belongs to class (i / 8) mod 8 and CTA class mod C at every
+// panel (the active rows shrink from the top, and the turns keep the shares
+// even). Each CTA sums V^H X over its classes, the eight class sums are added
+// in order (through distributed shared memory), so the result does not depend
+// on C, and each CTA updates its own rows. One CTA a mode left most SMs idle
+// with few modes, and the FP64 pipe of one SM bounds a block reflector (Q^H of a
+// transmission body, 37 modes of 268 x 222 with 8 columns: 1.05 ms on one CTA a
+// mode, 0.53 with C = 4).
+template <int TN, int C>
+struct BrRowSmem {
+  double2 P[C > 1 ? 2 : 1][8 / C][kNB][TN + 1];   // class sums, double-buffered over panels
+  double2 W[kNB][TN + 1];
+  double2 T[kNB][kNB + 1];
+};
+
+template <int TN, int C>
+__device__ void apply_block_reflector_rows(const double2 *__restrict__ A, int lda, int rows, int k0, int nbp,
+                                           const double2 *__restrict__ Tg, double2 *__restrict__ X, int ldx,
+                                           int ncols, BrRowSmem<TN, C> &sm, int p) {
+  constexpr int NT = kNB * TN;
+  const int rank = C > 1 ? (int)cg::this_cluster().block_rank() : 0, buf = C > 1 ? p & 1 : 0;
+  const int tid = threadIdx.x, ta = tid / TN, tc = tid % TN;
+  for (int e = tid; e < kNB * kNB; e += NT) sm.T[e % kNB][e / kNB] = Tg[e];
+  const int t0 = k0 / 8;                                  // the panel's first turn (k0 is a multiple of 16)
+  const int c = k0 + ta;
+  const double2 *va = A + (size_t)c * lda, *xc = X + (size_t)tc * ldx;
+#pragma unroll
+  for (int u = 0; u < 8 / C; ++u) {
+    double2 w = make_double2(0.0, 0.0), w1 = w;
+    if (ta < nbp && tc < ncols) {
+      for (int t = t0 + ((rank + C * u - t0) & 7); 8 * t < rows; t += 8) {
+        const int r0 = 8 * t, r1 = min(rows, r0 + 8);
+        if (r0 > c && r0 + 8 <= rows) {                   // whole turns below the diagonal
+#pragma unroll
+          for (int r = 0; r < 8; r += 2) {
+            w = cfma_conj(w, va[r0 + r], xc[r0 + r]);
+            w1 = cfma_conj(w1, va[r0 + r + 1], xc[r0 + r + 1]);
+          }
+        } else {
+          for (int r = max(r0, c); r < r1; ++r) {
+            if (r == c) w = cadd(w, xc[r]);
+            else w = cfma_conj(w, va[r], xc[r]);
+          }
+        }
+      }
+    }
+    sm.P[buf][u][ta][tc] = cadd(w, w1);
+  }
+  double2 w = make_double2(0.0, 0.0);
+  if constexpr (C > 1) {
+    cg::this_cluster().sync();
+#pragma unroll
+    for (int cl = 0; cl < 8; ++cl)
+      w = cadd(w, cg::this_cluster().map_shared_rank(&sm.P[buf][0][0][0], cl % C)[(cl / C * kNB + ta) * (TN + 1) + tc]);
+  } else {
+#pragma unroll
+    for (int cl = 0; cl < 8; ++cl) w = cadd(w, sm.P[0][cl][ta][tc]);     // this thread's own
+  }
+  sm.W[ta][tc] = w;
+  __syncthreads();
+  double2 wp = make_double2(0.0, 0.0);                    // W' = T^H W
+  for (int b = 0; b <= ta; ++b) wp = cfma_conj(wp, sm.T[b][ta], sm.W[b][tc]);
+  __syncthreads();
+  sm.W[ta][tc] = wp;
+  __syncthreads();
+  // X -= V W': one row and column an item, rows fastest
+  const int first = t0 + ((rank - t0) % C + C) % C;
+  const int turns = 8 * first < rows ? (rows - 8 * first + 8 * C - 1) / (8 * C) : 0;
+  for (int e = tid; e < turns * 8 * ncols; e += NT) {
+    const int q = e % (turns * 8), cc = e / (turns * 8);
+    const int i = 8 * (first + q / 8 * C) + q % 8;
+    if (i >= rows) continue;
+    double2 x = X[(size_t)cc * ldx + i];
+    if (i >= k0 + kNB && nbp == kNB) {
+#pragma unroll
+      for (int a = 0; a < kNB; ++a) x = cfms(x, A[(size_t)(k0 + a) * lda + i], sm.W[a][cc]);
+    } else {
+      for (int a = 0; a < nbp; ++a) x = cfms(x, vget(A, lda, rows, k0, nbp, i, a), sm.W[a][cc]);
+    }
+    X[(size_t)cc * ldx + i] = x;
+  }
+  __syncthreads();
+}
+
+// The next panel's columns of a mode: TN of them (blockIdx.y), rows over a cluster.
+template <int TN, int C>
+__global__ void __launch_bounds__(kNB * TN)
+qr_next_rows_kernel(const ObsDev *__restrict__ obs, const int *__restrict__ task_obs,
+                    const int *__restrict__ task_mode, int p) {
+  const int task = blockIdx.x / C;
+  const ObsDev &o = obs[task_obs[task]];
+  const int d = task_mode[task], k0 = p * kNB, nbp = min(kNB, o.cols - k0);
+  const int c0 = k0 + nbp + blockIdx.y * TN;
+  if (c0 >= o.cols) return;                               // uniform over the cluster
+  __shared__ BrRowSmem<TN, C> sm;
+  double2 *A = o.A + (size_t)d * o.cols * o.rows;
+  apply_block_reflector_rows<TN, C>(A, o.rows, o.rows, k0, nbp, o.T + ((size_t)d * o.npanels + p) * kNB * kNB,
+                                    A + (size_t)c0 * o.rows, o.rows, min(TN, o.cols - c0), sm, 0);
+  if constexpr (C > 1) cg::this_cluster().sync();         // the class sums are read by the whole cluster
+}
+
+// Q^H applied to TN right-hand-side columns of mode d (X_d is [2W][rows]
+// column-major), rows over a cluster; the panels are sequential, so
+// parallelism comes from modes x tiles x cluster.
+template <int TN, int C>
+__global__ void __launch_bounds__(kNB * TN)
+apply_qh_rows_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int ncols_total) {
   const ObsDev &o = *od;
-  const int d = blockIdx.x;
-  if (!owns_mode(o, d)) return;
-  const int c0 = blockIdx.y * kTA;
-  if (c0 >= ncols_total) return;
-  const int ncols = min(kTA, ncols_total - c0);
-  __shared__ BrSmem<kTA> sm;
+  const int d = blockIdx.x / C, c0 = blockIdx.y * TN;
+  if (!owns_mode(o, d) || c0 >= ncols_total) return;
+  __shared__ BrRowSmem<TN, C> sm;
   const double2 *A = o.A + (size_t)d * o.cols * o.rows;
   double2 *Xd = X + ((size_t)d * ncols_total + c0) * o.rows;
-  for (int p = 0; p < o.npanels; ++p) {
-    const int k0 = p * kNB;
-    const int nbp = min(kNB, o.cols - k0);
-    const double2 *Tg = o.T + ((size_t)d * o.npanels + p) * kNB * kNB;
-    apply_block_reflector_h<kTA>(A, o.rows, o.rows, k0, nbp, Tg, Xd, o.rows, ncols, sm);
-  }
+  for (int p = 0; p < o.npanels; ++p)
+    apply_block_reflector_rows<TN, C>(A, o.rows, o.rows, p * kNB, min(kNB, o.cols - p * kNB),
+                                      o.T + ((size_t)d * o.npanels + p) * kNB * kNB, Xd, o.rows,
+                                      min(TN, ncols_total - c0), sm, p);
+  if constexpr (C > 1) cg::this_cluster().sync();
 }
+
+constexpr int kTA = 8;    // columns of the narrow tiles
 
 // Blocked back substitution R X = Y on the first `cols` rows of each RHS
 // column (R real-diagonal upper triangle of the packed factors). One warp
 // per RHS column inside 32x32 diagonal blocks; rows above are updated with
 // the solved block before moving up.
 constexpr int kTB = 32;
-constexpr int kTS = 8;    // RHS columns per CTA in the triangular solve (one warp each)
+// kTS: RHS columns per CTA (one warp each in the diagonal blocks): 8, or 2 where
+// 8 would leave SMs idle (few modes times columns).
+template <int kTS>
 __global__ void __launch_bounds__(kThreads)
 trsm_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int ncols_total) {
   const ObsDev &o = *od;
@@ -846,10 +947,9 @@ bool panel_fits_one_cta(int rows) {
 template <int NT>
 cudaError_t launch_panel_nt(const ObsDev *d_obs, const int *d_task_obs, const int *d_task_mode,
                             int ntasks, int p, int max_panel_rows, int cluster, cudaStream_t st) {
-  const int sms = sm_count();
-  if (cluster == 4 || (cluster == 0 && 4 * ntasks <= sms))
+  if (cluster == 4)
     return launch_panel_cluster<4, NT>(d_obs, d_task_obs, d_task_mode, ntasks, p, max_panel_rows, st);
-  if (cluster == 2 || (cluster == 0 && 2 * ntasks <= sms))
+  if (cluster == 2)
     return launch_panel_cluster<2, NT>(d_obs, d_task_obs, d_task_mode, ntasks, p, max_panel_rows, st);
   if (!panel_fits_one_cta<NT>(max_panel_rows))   // the panel and the static arrays exceed one CTA
     return launch_panel_cluster<2, NT>(d_obs, d_task_obs, d_task_mode, ntasks, p, max_panel_rows, st);
@@ -874,18 +974,25 @@ cudaError_t launch_qr_panel(const ObsDev *d_obs, const int *d_task_obs, const in
     return cudaErrorInvalidConfiguration;                     // asked for, but it does not fit
   }
   if (max_panel_rows <= kPanelSmemRows) {
-    // threads 0 (auto): 256 when the panel runs on one CTA and has more than
-    // 128 rows (two warps per SM sub-partition hide the FP64 latency of the
-    // per-row sweep; in clusters the wider CTAs' exchanges cost more), else 128
+    // The automatic choice, from builds of N = 40 .. 360 proxies with 9 .. 91
+    // tasks, native and split (ms a build, this rule against the one that took
+    // as many CTAs a mode as fit one wave and 256 threads on one CTA):
+    //   up to 128 rows one CTA of 128 threads: a cluster's exchanges cost more
+    //     than a quarter of the rows saves (N = 60, 17 tasks: 0.67 against 0.73);
+    //   more rows, two CTAs a mode while they fit one wave, four above 224 rows
+    //     (N = 150, 33 tasks: 2.69 against 2.94; N = 240, 17 tasks, four: 5.1, two: 5.2);
+    //   else one CTA, of 256 threads (two warps per SM sub-partition hide the FP64
+    //     latency) up to 288 rows and one CTA per SM (N = 150, 91 tasks: 2.54
+    //     against 2.99 with 128), of 128 threads above (cup: 11.6 against 12.3) and
+    //     where SMs hold several (the 8 obstacles of a batch: 7.6 against 8.7).
     const int sms = sm_count();
-    const int c_auto = (cluster == 0 && 4 * ntasks <= sms) ? 4 : (cluster == 0 && 2 * ntasks <= sms) ? 2 : 1;
-    const int c_eff = cluster != 0 ? cluster : c_auto;
-    const bool wide = threads == 256 || (threads == 0 && c_eff == 1 && max_panel_rows > 128);
-    if (wide)
-      return launch_panel_nt<256>(d_obs, d_task_obs, d_task_mode, ntasks, p, max_panel_rows,
-                                  cluster, st);
-    return launch_panel_nt<kPanelThreads>(d_obs, d_task_obs, d_task_mode, ntasks, p,
-                                          max_panel_rows, cluster, st);
+    int c_eff = cluster, nt = threads;
+    if (c_eff == 0)
+      c_eff = max_panel_rows <= 128 ? 1 : 4 * ntasks <= sms && max_panel_rows > 224 ? 4 : 2 * ntasks <= sms ? 2 : 1;
+    if (nt == 0) nt = c_eff == 1 && max_panel_rows > 128 && max_panel_rows <= 288 && ntasks <= sms ? 256 : 128;
+    if (nt == 256)
+      return launch_panel_nt<256>(d_obs, d_task_obs, d_task_mode, ntasks, p, max_panel_rows, c_eff, st);
+    return launch_panel_nt<kPanelThreads>(d_obs, d_task_obs, d_task_mode, ntasks, p, max_panel_rows, c_eff, st);
   }
   qr_panel_kernel<<<ntasks, kThreads, 0, st>>>(d_obs, d_task_obs, d_task_mode, p);
   return cudaGetLastError();
@@ -894,17 +1001,65 @@ cudaError_t launch_qr_panel(const ObsDev *d_obs, const int *d_task_obs, const in
 // The next panel's kNB columns, in native FP64 with narrow tiles (two CTAs
 // per mode): this update is on the critical path of the factorisation, where
 // the split path would first need the panel's digits.
-cudaError_t launch_qr_update_next(const ObsDev *d_obs, const int *d_task_obs,
-                                  const int *d_task_mode, int ntasks, int p, cudaStream_t st) {
-  if (ntasks <= 0) return cudaSuccess;
-  static const bool carve = (prefer_max_shared(qr_update_kernel<kTA>), true);
-  (void)carve;
-  qr_update_kernel<kTA><<<dim3(ntasks, kNB / kTA), kNB * kTA, 0, st>>>(d_obs, d_task_obs,
-                                                                      d_task_mode, p, 0);
-  return cudaGetLastError();
+namespace {
+
+template <typename K, typename... Args>
+cudaError_t launch_clusters(K *kernel, dim3 grid, int threads, int C, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = C > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Columns from kNB past the panel onward, native FP64 or split digits.
+template <int TN>
+cudaError_t launch_qh_rows(const ObsDev *d_o, int D, double2 *X, int ncol, int C, cudaStream_t st) {
+  const unsigned tiles = (ncol + TN - 1) / TN;
+  if (C == 8) return launch_clusters(apply_qh_rows_kernel<TN, 8>, dim3(D * 8, tiles), kNB * TN, 8, st, d_o, X, ncol);
+  if (C == 4) return launch_clusters(apply_qh_rows_kernel<TN, 4>, dim3(D * 4, tiles), kNB * TN, 4, st, d_o, X, ncol);
+  if (C == 2) return launch_clusters(apply_qh_rows_kernel<TN, 2>, dim3(D * 2, tiles), kNB * TN, 2, st, d_o, X, ncol);
+  return launch_clusters(apply_qh_rows_kernel<TN, 1>, dim3(D, tiles), kNB * TN, 1, st, d_o, X, ncol);
+}
+
+// Native Q^H: rows over clusters while every CTA gets an SM of its own and two
+// turns of rows.
+cudaError_t launch_apply_qh_fp64(const ObsDev *d_o, const ObsDev &h, double2 *X, int ncol, cudaStream_t st) {
+  const int TN = ncol >= 8 ? 8 : ncol > 2 ? 4 : 2;
+  const int tiles = h.D * ((ncol + TN - 1) / TN);
+  int C = 1;
+  while (C < 8 && 2 * C * tiles <= sm_count() && 32 * C <= h.rows) C *= 2;
+  if (TN == 8) return launch_qh_rows<8>(d_o, h.D, X, ncol, C, st);
+  if (TN == 4) return launch_qh_rows<4>(d_o, h.D, X, ncol, C, st);
+  return launch_qh_rows<2>(d_o, h.D, X, ncol, C, st);
+}
+
+}  // namespace
+
+cudaError_t launch_qr_update_next(const ObsDev *d_obs, const int *d_task_obs,
+                                  const int *d_task_mode, int ntasks, int p, int rows, cudaStream_t st) {
+  if (ntasks <= 0) return cudaSuccess;
+  const int sms = sm_count();
+  if (8 * ntasks <= sms && rows >= 128)
+    return launch_clusters(qr_next_rows_kernel<kNB, 8>, dim3(ntasks * 8), kNB * kNB, 8, st, d_obs, d_task_obs,
+                           d_task_mode, p);
+  if (4 * ntasks <= sms && rows >= 64)
+    return launch_clusters(qr_next_rows_kernel<kNB, 4>, dim3(ntasks * 4), kNB * kNB, 4, st, d_obs, d_task_obs,
+                           d_task_mode, p);
+  if (2 * ntasks <= sms)
+    return launch_clusters(qr_next_rows_kernel<kNB, 2>, dim3(ntasks * 2), kNB * kNB, 2, st, d_obs, d_task_obs,
+                           d_task_mode, p);
+  static const bool carve = (prefer_max_shared(qr_next_rows_kernel<kTA, 1>), true);
+  (void)carve;
+  return launch_clusters(qr_next_rows_kernel<kTA, 1>, dim3(ntasks, kNB / kTA), kNB * kTA, 1, st, d_obs, d_task_obs,
+                         d_task_mode, p);
+}
 cudaError_t launch_qr_update_rest(const ObsDev *d_obs, const int *d_task_obs,
                                   const int *d_task_mode, int ntasks, int p, int slices,
                                   int max_rest_cols, int rest_grid, bool use_y, cudaStream_t st) {
@@ -917,6 +1072,17 @@ cudaError_t launch_qr_update_rest(const ObsDev *d_obs, const int *d_task_obs,
                                   (max_rest_cols + split_update_tile_cols() - 1) /
                                       split_update_tile_cols(),
                                   split_update_tile_cols(), rest_grid == 1, use_y, st);
+  // tiles of 4 or 8 columns where 16 would leave SMs idle or the last wave short
+  const long long t16 = (long long)ntasks * ((max_rest_cols + kTN - 1) / kTN);
+  if (t16 < 8LL * sm_count()) {
+    if (t16 < 2LL * sm_count())
+      qr_update_kernel<4><<<dim3(ntasks, (max_rest_cols + 3) / 4), kNB * 4, 0, st>>>(d_obs, d_task_obs, d_task_mode,
+                                                                                     p, kNB);
+    else
+      qr_update_kernel<kTA><<<dim3(ntasks, (max_rest_cols + kTA - 1) / kTA), kNB * kTA, 0, st>>>(
+          d_obs, d_task_obs, d_task_mode, p, kNB);
+    return cudaGetLastError();
+  }
   static const bool carve = (prefer_max_shared(qr_update_kernel<kTN>), true);
   (void)carve;
   qr_update_kernel<kTN><<<dim3(ntasks, (max_rest_cols + kTN - 1) / kTN), kThreads, 0, st>>>(
@@ -951,8 +1117,7 @@ cudaError_t launch_apply(const ObsDev *d_o, const ObsDev &h, int W, const double
   if (h.slices > 0 && W >= kSplitApplyMinWaves) {
     e = launch_apply_qh_split(d_o, h, X, ncol, digit_scratch, st);
   } else {
-    apply_qh_kernel<<<dim3(h.D, (ncol + kTA - 1) / kTA), kNB * kTA, 0, st>>>(d_o, X, ncol);
-    e = cudaGetLastError();
+    e = launch_apply_qh_fp64(d_o, h, X, ncol, st);
   }
   prof_end(pid, st, rhs * (16.0 * h.rows * h.cols - 8.0 * h.cols * h.cols));
   if (e != cudaSuccess) return e;
@@ -962,7 +1127,10 @@ cudaError_t launch_apply(const ObsDev *d_o, const ObsDev &h, int W, const double
   } else if (h.slices > 0) {
     e = launch_trsm_split(d_o, h, X, ncol, st);
   } else {
-    trsm_kernel<<<dim3(h.D, (ncol + kTS - 1) / kTS), kThreads, 0, st>>>(d_o, X, ncol);
+    if (h.D * ((ncol + 7) / 8) >= sm_count())
+      trsm_kernel<8><<<dim3(h.D, (ncol + 7) / 8), kThreads, 0, st>>>(d_o, X, ncol);
+    else
+      trsm_kernel<2><<<dim3(h.D, (ncol + 1) / 2), kThreads, 0, st>>>(d_o, X, ncol);
     e = cudaGetLastError();
   }
   prof_end(pid, st, rhs * 4.0 * h.cols * h.cols);
