@@ -210,10 +210,11 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
  *                   updates, FP64 scalars; one CTA per mode, so with
  *                   panel_cluster 0 or 1; the build fails with AXI_ERR_CUDA
  *                   where a panel does not fit one CTA);
- *   "rest_start"    0 each step's trailing update starts as soon as the
- *                   panel (and its digits) is done, beside the next-panel
- *                   update; 1 it starts after the next-panel update, so that
- *                   it runs beside the next panel only;
+ *   "rest_start"    0 auto: under stream capture each step's trailing update
+ *                   starts as soon as the panel (and its digits) is done,
+ *                   beside the next-panel update; launched directly it starts
+ *                   after the next-panel update, so that it runs beside the
+ *                   next panel only; 1 always after the next-panel update;
  *   "apply_cluster" split plans' Q^H in axi_apply_operator: 0 auto (4 CTAs
  *                   per (mode, 32-column tile) when all of them fit in one
  *                   wave of two CTAs per SM, else 2), or 2, 4.
@@ -225,9 +226,8 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
  * 1..100; it synchronises the stream, so not under stream capture): first
  * the panel chain's choices together, then, for split plans, the next-panel
  * update's cluster, the fixed-point panel (128 and 256 threads) and the fill
- * chunk, each with the best so far ("rest_start" is left as given: its two
- * settings time alike with direct launches, but 1 is slower in a CUDA
- * graph). It keeps the fastest in the plan, rebuilds the
+ * chunk, each with the best so far ("rest_start" is left as given: 1 is
+ * slower in a CUDA graph). It keeps the fastest in the plan, rebuilds the
  * operator with it and, when json_out is
  * not NULL, writes the choice with its build time ("build_ms"), the number
  * of candidates timed and the number skipped because they cannot run on this
