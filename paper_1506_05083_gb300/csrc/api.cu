@@ -25,38 +25,42 @@ struct ObsHost {
   ObsDev dev;  // device pointers are filled at build time from the offsets below
   std::vector<double> coll, src, srcx, tab_cos, tab_s2;
   std::vector<double2> tw_P;
-  std::vector<int> fft_perm, fft_perm_q;
+  std::vector<int> fft_perm, fft_perm_q[3];
   std::vector<double2> tw_q;
   size_t off_coll, off_src, off_srcx, off_cos, off_s2, off_tw, off_A, off_tau, off_T;
   size_t off_ring = 0;
   std::vector<double2> tab_ring;
   size_t off_svdU = 0, off_svdV = 0, off_svdS = 0, off_svdSw = 0, off_svdPerm = 0;
   size_t off_ybuf = 0, off_ykey = 0, off_ydig = 0, off_yexp = 0;
-  size_t off_vdig = 0, off_vexp = 0, off_ckey = 0, off_rdig = 0, off_rex = 0, off_perm = 0, off_perm_q = 0, off_tw_q = 0;
-  std::vector<unsigned short> fill_cdig;   // split fill: cos-table digits [S][2 MR][Lp]
+  size_t off_vdig = 0, off_vexp = 0, off_ckey = 0, off_rdig = 0, off_rex = 0, off_perm = 0, off_perm_q[3] = {0, 0, 0}, off_tw_q = 0;
+  std::vector<unsigned short> fill_cdig[3];   // split fill: cos-table digits [S][2 MR][Lp] per stride class
   std::vector<int> fill_cex;               // and row exponents [2 MR]
-  size_t off_fcdig = 0, off_fcex = 0;
+  size_t off_fcdig[3] = {0, 0, 0}, off_fcex = 0;
+  std::vector<int> fill_list;              // pairs by proxy set and stride class
+  size_t off_flist = 0;
   std::vector<unsigned char> fill_sig;     // [2][M][N] sub-grid stride per ring pair
   size_t off_fsig = 0;
   std::vector<unsigned char> owned;        // [D] modes this process factors (axi_plan_shard)
   size_t off_owned = 0;
 };
 
-// Digits of the folded cosine table of the split fill (fill_mma.cu): row
-// r < 2 MR holds mode n = 2 (r mod MR) + r / MR, entries w_l cos(2 pi n l / q)
-// for l < L (w_0 = 1, else 2), zero elsewhere; balanced base-128 digits of
-// round(x 2^{7S - e}) with e the row's exponent (|x| < 2^e).
-void fill_cos_digits(ObsHost &h, int S) {
+// Digits of the folded cosine table of the split fill (fill_mma.cu) for stride
+// class c: row r < 2 MR holds mode n = 2 (r mod MR) + r / MR, entries
+// w_i cos(2 pi n l / q), l = i << c, for i < L (w_0 = 1, else 2), zero elsewhere;
+// balanced base-128 digits of round(x 2^{7S - e}) with e the row's exponent
+// over every l of the folded range (|x| < 2^e; the same for all classes).
+void fill_cos_digits(ObsHost &h, int S, int c) {
   const ObsDev &d = h.dev;
-  const int q = d.q, rows = 2 * d.fill_MR, Lp = d.fill_Lp, L = d.fill_L;
-  h.fill_cdig.assign((size_t)S * rows * Lp, 0);
+  const int q = d.q, rows = 2 * d.fill_MR, Lp = d.fill_Lp[c], L = d.fill_L[c];
+  std::vector<unsigned short> &dig = h.fill_cdig[c];
+  dig.assign((size_t)S * rows * Lp, 0);
   h.fill_cex.assign(rows, 0);
-  std::vector<double> v(L);
+  std::vector<double> v(d.fill_L[0]);
   for (int r = 0; r < rows; ++r) {
     const int n = 2 * (r % d.fill_MR) + r / d.fill_MR;
     if (n >= d.D) continue;
     double mx = 0.0;
-    for (int l = 0; l < L; ++l) {
+    for (int l = 0; l < d.fill_L[0]; ++l) {
       v[l] = (l == 0 ? 1.0 : 2.0) * h.tab_cos[(size_t)n * l % q];
       if ((n & 1) && 2 * l == q / 2) v[l] = 0.0;          // cos(pi n / 2) = 0 for odd n
       mx = std::max(mx, std::fabs(v[l]));
@@ -64,8 +68,8 @@ void fill_cos_digits(ObsHost &h, int S) {
     if (mx == 0.0) continue;
     const int e = std::ilogb(mx) + 1;
     h.fill_cex[r] = e;
-    for (int l = 0; l < L; ++l) {
-      long long m = std::llround(std::ldexp(v[l], 7 * S - e));
+    for (int i = 0; i < L; ++i) {
+      long long m = std::llround(std::ldexp(v[(size_t)i << c], 7 * S - e));
       for (int s = S; s >= 1; --s) {
         int dg;
         if (s > 1) {
@@ -78,17 +82,17 @@ void fill_cos_digits(ObsHost &h, int S) {
         const float f = (float)dg;
         uint32_t b;
         std::memcpy(&b, &f, sizeof(b));
-        h.fill_cdig[((size_t)(s - 1) * rows + r) * Lp + l] = (unsigned short)(b >> 16);
+        dig[((size_t)(s - 1) * rows + r) * Lp + i] = (unsigned short)(b >> 16);
       }
     }
   }
-  if (!d.fill_tc) return;
+  if (!d.fill_tc[c]) return;
   // tcgen05 layout: per (parity, 16-row chunk of the contraction, digit) one
   // K-major no-swizzle tile of MR rows x 16 k (core matrices of 8 rows x 8 k,
   // 128 bytes apart along k, 256 bytes apart along rows), so that one bulk
   // copy brings a chunk's tiles of all digits
   const int MR = d.fill_MR, nch = Lp / 16;
-  std::vector<unsigned short> tcl(h.fill_cdig.size(), 0);
+  std::vector<unsigned short> tcl(dig.size(), 0);
   for (int part = 0; part < 2; ++part)
     for (int ch = 0; ch < nch; ++ch)
       for (int s = 0; s < S; ++s)
@@ -96,9 +100,34 @@ void fill_cos_digits(ObsHost &h, int S) {
           for (int kk = 0; kk < 16; ++kk) {
             const size_t tile = ((size_t)(part * nch + ch) * S + s) * MR * 16;
             const size_t in = (size_t)(r / 8) * 128 + (kk / 8) * 64 + (r % 8) * 8 + (kk % 8);
-            tcl[tile + in] = h.fill_cdig[((size_t)s * rows + part * MR + r) * Lp + ch * 16 + kk];
+            tcl[tile + in] = dig[((size_t)s * rows + part * MR + r) * Lp + ch * 16 + kk];
           }
-  h.fill_cdig.swap(tcl);
+  dig.swap(tcl);
+}
+
+// The split fill's pairs by proxy set and stride class. A class whose pairs
+// would save less than its launches cost joins the next finer one, where its
+// skipped nodes stay zero: about 0.08 ns a pair and folded node against 30 us.
+void fill_classes(ObsHost &h, int MN, int sets) {
+  ObsDev &d = h.dev;
+  for (int e = 0; e < sets; ++e) {
+    const unsigned char *sig = h.fill_sig.data() + (size_t)e * MN;
+    int cnt[3] = {0, 0, 0}, to[3] = {0, 1, 2};
+    for (int p = 0; p < MN; ++p) cnt[sig[p] >> 1]++;      // strides 1, 2, 4
+    for (int c = 2; c >= 1; --c)
+      if ((double)cnt[c] * (d.fill_L[c - 1] - d.fill_L[c]) < 400000.0) {
+        cnt[c - 1] += cnt[c];
+        for (int u = c; u < 3; ++u)
+          if (to[u] == c) to[u] = c - 1;
+        cnt[c] = 0;
+      }
+    for (int c = 0; c < 3; ++c) {
+      d.fill_off[e][c] = (int)h.fill_list.size();
+      for (int p = 0; p < MN; ++p)
+        if (to[sig[p] >> 1] == c) h.fill_list.push_back(p);
+      d.fill_cnt[e][c] = (int)h.fill_list.size() - d.fill_off[e][c];
+    }
+  }
 }
 
 // Sub-grid strides of the fill (axi_fill_subgrid per proxy set); `full`
@@ -504,11 +533,14 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
     // radices 4, 2, 3, 5 and output permutations for the FFTs of length P
     // (apply) and q (fill)
     d.fft_nst = fft_plan(o.P, d.fft_rad, h.fft_perm);
-    d.fft_nst_q = fft_plan(o.q, d.fft_rad_q, h.fft_perm_q, d.D, &d.fft_sum_last_q);
+    for (int c = 0; c < 3; ++c)             // q >> c nodes, where that stride divides q / 2
+      d.fft_nst_q[c] = (o.q / 2) % (1 << c) == 0 && (o.q >> c) >= d.D
+                           ? fft_plan(o.q >> c, d.fft_rad_q[c], h.fft_perm_q[c], d.D, &d.fft_sum_last_q[c])
+                           : 0;
     h.tw_q.resize(o.q);
     for (int r = 0; r < o.q; ++r)
       h.tw_q[r] = make_double2(std::cos(2.0 * kPi * r / o.q), -std::sin(2.0 * kPi * r / o.q));
-    h.off_perm_q = off; off = align_up(off + sizeof(int) * h.fft_perm_q.size());
+    for (int c = 0; c < 3; ++c) { h.off_perm_q[c] = off; off = align_up(off + sizeof(int) * h.fft_perm_q[c].size()); }
     h.off_tw_q = off; off = align_up(off + sizeof(double2) * h.tw_q.size());
     h.off_coll = off; off = align_up(off + sizeof(double) * h.coll.size());
     h.off_perm = off; off = align_up(off + sizeof(int) * h.fft_perm.size());
@@ -555,23 +587,35 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
       h.off_yexp = off; off = align_up(off + sizeof(int) * (size_t)d.D * 2 * axi::kNB);
       h.off_rdig = off; off = align_up(off + axi::r_digit_bytes(d));
       h.off_rex = off; off = align_up(off + axi::r_exponent_bytes(d));
-      // split fill: folded length, padding, cos-table digits, pair chunk
-      const int hh = d.q / 2;
-      d.fill_L = (hh % 2 == 0) ? hh / 2 + 1 : (hh + 1) / 2;
-      d.fill_Lp = (d.fill_L + 31) / 32 * 32;
+      // split fill: folded lengths, padding, cos-table digits, pair lists, scratch
       d.fill_MR = ((d.D + 1) / 2 + 15) / 16 * 16;
-      d.fill_tc = axi::fill_uses_tc(d.fill_Lp, d.fill_MR) ? 1 : 0;
-      const int kinds = o.bc == AXI_BC_TRANSMISSION ? 4 : 1;
-      const size_t per_pair = (size_t)2 * 2 * kinds * axi::kFillDigits * d.fill_Lp * sizeof(unsigned short);
-      const size_t cap = (size_t)512 << 20;
-      d.fill_chunk_pairs = (int)std::max<size_t>(8, std::min<size_t>((size_t)o.M * o.N, cap / per_pair));
-      // the tcgen05 layout pads the columns to whole 128-column tiles
-      const size_t pad = d.fill_tc ? (size_t)2 * 128 * axi::kFillDigits * d.fill_Lp * sizeof(unsigned short) : 0;
-      fill_gdig_bytes = std::max(fill_gdig_bytes, per_pair * d.fill_chunk_pairs + pad);
-      fill_gex_bytes = std::max(fill_gex_bytes, sizeof(int) * 2 * 2 * kinds * (size_t)d.fill_chunk_pairs);
-      fill_cos_digits(h, axi::kFillDigits);
-      h.off_fcdig = off; off = align_up(off + sizeof(unsigned short) * h.fill_cdig.size());
+      for (int c = 0; c < 3; ++c) {
+        const int hh = (d.q / 2) >> c;
+        d.fill_L[c] = (hh % 2 == 0) ? hh / 2 + 1 : (hh + 1) / 2;
+        d.fill_Lp[c] = (d.fill_L[c] + 31) / 32 * 32;
+        d.fill_tc[c] = axi::fill_uses_tc(d.fill_Lp[c], d.fill_MR) ? 1 : 0;
+      }
+      const int sets = o.bc == AXI_BC_TRANSMISSION ? 2 : 1;
+      fill_classes(h, o.M * o.N, sets);
+      // sample digits of the largest chunk any class asks for, up to 512 MB and a
+      // pad: the tcgen05 layout rounds the columns up to whole 128-column tiles
+      d.fill_cap = 0;
+      for (int e = 0; e < sets; ++e)
+        for (int c = 0; c < 3; ++c) {
+          if (d.fill_cnt[e][c] == 0) continue;
+          const size_t per_pair = axi::fill_pair_bytes(d, c);
+          const size_t pairs = std::max<size_t>(
+              8, std::min<size_t>((size_t)d.fill_cnt[e][c], ((size_t)512 << 20) / per_pair));
+          d.fill_cap = std::max(d.fill_cap, pairs * per_pair + axi::fill_pad_bytes(d, c));
+        }
+      fill_gdig_bytes = std::max(fill_gdig_bytes, d.fill_cap);
+      fill_gex_bytes = std::max(fill_gex_bytes, sizeof(int) * 4 * sets * (size_t)o.M * o.N);
+      for (int c = 0; c < 3; ++c) {
+        if (d.fill_cnt[0][c] + d.fill_cnt[1][c] > 0) fill_cos_digits(h, axi::kFillDigits, c);
+        h.off_fcdig[c] = off; off = align_up(off + sizeof(unsigned short) * h.fill_cdig[c].size());
+      }
       h.off_fcex = off; off = align_up(off + sizeof(int) * h.fill_cex.size());
+      h.off_flist = off; off = align_up(off + sizeof(int) * h.fill_list.size());
     }
   }
   if (fill_gdig_bytes > 0) {
@@ -836,7 +880,7 @@ axi_status axi_build_operator(axi_plan *plan, void *d_workspace, size_t bytes, v
     d.fill_sig = reinterpret_cast<const unsigned char *>(ws + h.off_fsig);
     d.mode_owned = reinterpret_cast<const unsigned char *>(ws + h.off_owned);
     d.fft_perm = reinterpret_cast<const int *>(ws + h.off_perm);
-    d.fft_perm_q = reinterpret_cast<const int *>(ws + h.off_perm_q);
+    for (int c = 0; c < 3; ++c) d.fft_perm_q[c] = reinterpret_cast<const int *>(ws + h.off_perm_q[c]);
     d.tw_q = reinterpret_cast<const double2 *>(ws + h.off_tw_q);
     d.A = reinterpret_cast<double2 *>(ws + h.off_A);
     d.tau = reinterpret_cast<double2 *>(ws + h.off_tau);
@@ -856,7 +900,8 @@ axi_status axi_build_operator(axi_plan *plan, void *d_workspace, size_t bytes, v
     d.yexp = d.slices > 0 ? reinterpret_cast<int *>(ws + h.off_yexp) : nullptr;
     d.rex = d.slices > 0 ? reinterpret_cast<int *>(ws + h.off_rex) : nullptr;
     if (d.slices > 0) {
-      d.fill_cdig = reinterpret_cast<const unsigned short *>(ws + h.off_fcdig);
+      for (int c = 0; c < 3; ++c) d.fill_cdig[c] = reinterpret_cast<const unsigned short *>(ws + h.off_fcdig[c]);
+      d.fill_list = reinterpret_cast<const int *>(ws + h.off_flist);
       d.fill_cex = reinterpret_cast<const int *>(ws + h.off_fcex);
       d.fill_gdig = reinterpret_cast<uint32_t *>(ws + plan->off_fgdig);
       d.fill_gex = reinterpret_cast<int *>(ws + plan->off_fgex);
@@ -874,9 +919,14 @@ axi_status axi_build_operator(axi_plan *plan, void *d_workspace, size_t bytes, v
         {h.off_fsig, h.fill_sig.data(), h.fill_sig.size()},
         {h.off_owned, h.owned.data(), h.owned.size()},
         {h.off_perm, h.fft_perm.data(), sizeof(int) * h.fft_perm.size()},
-        {h.off_perm_q, h.fft_perm_q.data(), sizeof(int) * h.fft_perm_q.size()},
+        {h.off_perm_q[0], h.fft_perm_q[0].data(), sizeof(int) * h.fft_perm_q[0].size()},
+        {h.off_perm_q[1], h.fft_perm_q[1].data(), sizeof(int) * h.fft_perm_q[1].size()},
+        {h.off_perm_q[2], h.fft_perm_q[2].data(), sizeof(int) * h.fft_perm_q[2].size()},
         {h.off_tw_q, h.tw_q.data(), sizeof(double2) * h.tw_q.size()},
-        {h.off_fcdig, h.fill_cdig.data(), sizeof(unsigned short) * h.fill_cdig.size()},
+        {h.off_fcdig[0], h.fill_cdig[0].data(), sizeof(unsigned short) * h.fill_cdig[0].size()},
+        {h.off_fcdig[1], h.fill_cdig[1].data(), sizeof(unsigned short) * h.fill_cdig[1].size()},
+        {h.off_fcdig[2], h.fill_cdig[2].data(), sizeof(unsigned short) * h.fill_cdig[2].size()},
+        {h.off_flist, h.fill_list.data(), sizeof(int) * h.fill_list.size()},
         {h.off_fcex, h.fill_cex.data(), sizeof(int) * h.fill_cex.size()},
     };
     for (auto &c : cp) {
@@ -1263,7 +1313,7 @@ axi_status axi_operator_autotune(axi_operator *op, int32_t reps, void *stream, c
       }
     }
   }
-  if (s == AXI_OK && split && p->obs[0].dev.fill_cdig != nullptr) {
+  if (s == AXI_OK && split && p->obs[0].dev.fill_list != nullptr) {
     const axi::Tuning base = best;
     for (int fc : {0, 256, 128, 96, 64}) {
       if (fc == base.fill_chunk_mb) continue;

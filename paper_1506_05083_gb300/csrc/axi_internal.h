@@ -100,17 +100,23 @@ struct ObsDev {
   unsigned long long *ykey;
   unsigned short *ydig;
   int *yexp;
-  // split precision only: the fill's transform as a digit GEMM (fill_mma.cu).
-  // Folded length L, padded Lp (multiple of 32), MR rows per parity part;
-  // cos-table digits [kFillDigits][2 MR][Lp] and row exponents [2 MR];
-  // sample-digit scratch for fill_chunk_pairs ring pairs at a time.
-  int fill_L, fill_Lp, fill_MR, fill_chunk_pairs;
-  int fill_tc;            // 1: tcgen05 transform (fill_uses_tc), digit tiles in its layout
-  int apply_cluster;      // host side only: Tuning::apply_cluster for the split Q^H launch
-  const unsigned short *fill_cdig;
+  // split precision only: the fill's transform as a digit GEMM (fill_mma.cu),
+  // per stride class c = 0, 1, 2 (ring pairs sampled on every (1 << c)-th node):
+  // folded length L, padded Lp (multiple of 32), whether the transform runs on
+  // tcgen05 (fill_uses_tc) with the digit tiles in its layout, cos-table digits
+  // [kFillDigits][2 MR][Lp]; MR rows per parity part, row exponents [2 MR] of all
+  // classes. The pairs of proxy set e (interior, exterior) and class c are
+  // fill_list[fill_off[e][c] .. + fill_cnt[e][c]). Scratch for the sample
+  // digits of one chunk of pairs (fill_cap bytes) and all their exponents.
+  int fill_L[3], fill_Lp[3], fill_tc[3], fill_MR;
+  const unsigned short *fill_cdig[3];
   const int *fill_cex;
+  const int *fill_list;
+  int fill_off[2][3], fill_cnt[2][3];
+  size_t fill_cap;
   uint32_t *fill_gdig;
   int *fill_gex;
+  int apply_cluster;      // host side only: Tuning::apply_cluster for the split Q^H launch
   // truncated-SVD plans (AXI_PLAN_TSVD): R = U_R Sigma V^H per mode
   int tsvd;
   double2 *svdU, *svdV;   // [D][cols][cols] column-major
@@ -120,10 +126,13 @@ struct ObsDev {
   int fft_nst;            // radices of P for the apply's FFTs (0: P has other prime factors)
   int fft_rad[8];
   const int *fft_perm;    // [P] position of output n after the in-place FFT
-  int fft_nst_q;          // radices of q for the fill's FFT (0: direct cosine sums)
-  int fft_sum_last_q;     // 1: the needed modes are sums over the last stage's blocks
-  int fft_rad_q[8];
-  const int *fft_perm_q;  // [q]
+  // the fill's FFTs of q >> c nodes, c = 0, 1, 2: radices (0 stages: direct
+  // cosine sums, or a stride that does not divide q / 2), whether the needed
+  // modes are sums over the last stage's blocks, output positions [q >> c]
+  int fft_nst_q[3];
+  int fft_sum_last_q[3];
+  int fft_rad_q[3][8];
+  const int *fft_perm_q[3];
   const double2 *tw_q;    // [q] e^{-2 pi i r / q}
   // host side only: centre on the axis of the smallest sphere around targets
   // and interior proxies, the proxies' and targets' radii about it, and the
@@ -164,6 +173,15 @@ int *operator_status_word(const axi_operator *op);
 // accumulators of one parity fit tensor memory (MR <= 64 modes).
 constexpr int kFillTcMaxLp = 448;
 inline bool fill_uses_tc(int Lp, int MR) { return Lp <= kFillTcMaxLp && MR <= 64; }
+
+// Bytes of sample digits of a pair of stride class c (its one or two kinds:
+// two parities, real and imaginary columns), and of the tcgen05 layout's padding.
+inline size_t fill_pair_bytes(const ObsDev &h, int c) {
+  return (size_t)2 * 2 * (h.bc == AXI_BC_TRANSMISSION ? 2 : 1) * kFillDigits * h.fill_Lp[c] * sizeof(unsigned short);
+}
+inline size_t fill_pad_bytes(const ObsDev &h, int c) {
+  return h.fill_tc[c] ? (size_t)2 * 128 * kFillDigits * h.fill_Lp[c] * sizeof(unsigned short) : 0;
+}
 
 // Rows of R above 32-column block b, rounded up to 64, and their running
 // total over blocks 0..b-1 (sum of 64 ceil(j/2) for j < b = 64 floor(b^2/4)).

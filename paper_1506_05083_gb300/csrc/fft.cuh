@@ -8,7 +8,8 @@
 // position pos(n) holds X[n], where
 //   pos(n) = (n mod r_1) (P / r_1) + pos'(n div r_1)
 // recursively over the remaining radices (the table `perm` stores pos).
-// Twiddles come from the table tw[r] = e^{-2 pi i r / P}.
+// Twiddles come from the table tw[r tws] = e^{-2 pi i r / P} (tws > 1: a longer
+// sequence's table).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -26,7 +27,7 @@ __device__ __forceinline__ double2 c_mul_mi(double2 a) { return make_double2(a.y
 
 // In-place forward DFT X[n] = sum_l a[l] e^{-2 pi i n l / P}; output in digit-reversed order.
 __device__ __forceinline__ void warp_fft(double2 *a, int P, const double2 *__restrict__ tw, const int *rad, int nst,
-                         int lane) {
+                         int lane, int tws = 1) {
   int L = P;
   for (int s = 0; s < nst; ++s) {
     const int r = rad[s];
@@ -42,13 +43,13 @@ __device__ __forceinline__ void warp_fft(double2 *a, int P, const double2 *__res
         const double2 t3 = c_mul_mi(c_sub(x1, x3));
         const double2 y0 = c_add(t0, t2), y2 = c_sub(t0, t2), y1 = c_add(t1, t3), y3 = c_sub(t1, t3);
         x[0] = y0;
-        x[Lr] = c_mul(y1, tw[(j * 1 * stride_tw) % P]);
-        x[2 * Lr] = c_mul(y2, tw[(j * 2 * stride_tw) % P]);
-        x[3 * Lr] = c_mul(y3, tw[(j * 3 * stride_tw) % P]);
+        x[Lr] = c_mul(y1, tw[(j * 1 * stride_tw) % P * tws]);
+        x[2 * Lr] = c_mul(y2, tw[(j * 2 * stride_tw) % P * tws]);
+        x[3 * Lr] = c_mul(y3, tw[(j * 3 * stride_tw) % P * tws]);
       } else if (r == 2) {
         const double2 x0 = x[0], x1 = x[Lr];
         x[0] = c_add(x0, x1);
-        x[Lr] = c_mul(c_sub(x0, x1), tw[(j * stride_tw) % P]);
+        x[Lr] = c_mul(c_sub(x0, x1), tw[(j * stride_tw) % P * tws]);
       } else if (r == 3) {
         // w3 = e^{-2 pi i / 3} = -1/2 - i sqrt(3)/2
         const double h = 0.86602540378443864676;
@@ -58,8 +59,8 @@ __device__ __forceinline__ void warp_fft(double2 *a, int P, const double2 *__res
         const double2 m = make_double2(x0.x - 0.5 * s12.x, x0.y - 0.5 * s12.y);
         const double2 rot = make_double2(h * d12.y, -h * d12.x);     // -i sqrt(3)/2 (x1 - x2)
         x[0] = y0;
-        x[Lr] = c_mul(c_add(m, rot), tw[(j * stride_tw) % P]);
-        x[2 * Lr] = c_mul(c_sub(m, rot), tw[(j * 2 * stride_tw) % P]);
+        x[Lr] = c_mul(c_add(m, rot), tw[(j * stride_tw) % P * tws]);
+        x[2 * Lr] = c_mul(c_sub(m, rot), tw[(j * 2 * stride_tw) % P * tws]);
       } else {  // r == 5
         const double c1 = 0.30901699437494742410, c2 = -0.80901699437494742410;  // cos 2pi/5, cos 4pi/5
         const double s1 = 0.95105651629515357212, s2 = 0.58778525229247312917;   // sin 2pi/5, sin 4pi/5
@@ -73,10 +74,10 @@ __device__ __forceinline__ void warp_fft(double2 *a, int P, const double2 *__res
         const double2 n1 = make_double2(s1 * b1.y + s2 * b2.y, -(s1 * b1.x + s2 * b2.x));
         const double2 n2 = make_double2(s2 * b1.y - s1 * b2.y, -(s2 * b1.x - s1 * b2.x));
         x[0] = y0;
-        x[Lr] = c_mul(c_add(m1, n1), tw[(j * 1 * stride_tw) % P]);
-        x[2 * Lr] = c_mul(c_add(m2, n2), tw[(j * 2 * stride_tw) % P]);
-        x[3 * Lr] = c_mul(c_sub(m2, n2), tw[(j * 3 * stride_tw) % P]);
-        x[4 * Lr] = c_mul(c_sub(m1, n1), tw[(j * 4 * stride_tw) % P]);
+        x[Lr] = c_mul(c_add(m1, n1), tw[(j * 1 * stride_tw) % P * tws]);
+        x[2 * Lr] = c_mul(c_add(m2, n2), tw[(j * 2 * stride_tw) % P * tws]);
+        x[3 * Lr] = c_mul(c_sub(m2, n2), tw[(j * 3 * stride_tw) % P * tws]);
+        x[4 * Lr] = c_mul(c_sub(m1, n1), tw[(j * 4 * stride_tw) % P * tws]);
       }
     }
     __syncwarp();

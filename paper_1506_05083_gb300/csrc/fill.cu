@@ -140,23 +140,38 @@ fill_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict__ ou
   if (bad) atomicOr(o.status, kStatNonFinite);
 }
 
-// FFT variant (q = 2^a 3^b 5^c): one warp per (m, j) pair evaluates the
-// q/2 + 1 samples, mirrors them into the full even sequence of length q and
+__device__ const long long g_fill_ring_q62[trig::kRingTab][2] = {
+#include "ring_table_q62.inc"
+};
+
+__device__ __forceinline__ void fill_sincos(double x, double *sn, double *cs) {
+  if (fabs(x) < 1048576.0)
+    trig::sincos_ring_q(x, reinterpret_cast<const longlong2 *>(g_fill_ring_q62), sn, cs);
+  else
+    sincos(x, sn, cs);
+}
+
+// FFT variant (q = 2^a 3^b 5^c): one warp per (m, j) pair evaluates the samples
+// of its sub-grid (nodes l = 0, sg, 2 sg, .., i.e. the trapezoid rule on qs =
+// q / sg nodes), mirrors them into the full even sequence of length qs and
 // transforms it in shared memory with the mixed-radix warp FFT (fft.cuh):
-//   A_n = (1/q) sum_{l=0}^{q-1} g_l e^{-2 pi i n l / q},  n = 0 .. D-1.
-// Per sample this costs ~5 log2(q) FP64 operations instead of 2 D FMAs.
+//   A_n = (1/qs) sum_{i=0}^{qs-1} g_{i sg} e^{-2 pi i n i / qs},  n = 0 .. D-1.
+// Per sample this costs ~5 log2(qs) FP64 operations instead of 2 D FMAs. The
+// FP64 pipe bounds it; sin and cos run in fixed point, and the transform has
+// the pair's own length (with q nodes for every pair, the others zero, and FP64
+// table sincos the transmission body of 134 x 111 pairs, P = 72, took 1.93 ms,
+// now 0.97 ms).
 __global__ void __launch_bounds__(256)
 fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict__ out,
                 int ld_rows, int ld_cols) {
   const ObsDev &o = obs_arr[oi];
-  const int q = o.q, half = q / 2, D = o.D;
+  const int q = o.q, D = o.D;
   const int nw = blockDim.x >> 5;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   extern __shared__ double2 fsm[];
   double2 *tw = fsm;                                        // [q]
-  int *perm = reinterpret_cast<int *>(fsm + q);             // [q]
-  double2 *seq = fsm + q + (q + 1) / 2 + warp * q;          // [nw][q]
-  for (int i = threadIdx.x; i < q; i += blockDim.x) { tw[i] = o.tw_q[i]; perm[i] = o.fft_perm_q[i]; }
+  double2 *seq = fsm + q + warp * q;                        // [nw][q]
+  for (int i = threadIdx.x; i < q; i += blockDim.x) tw[i] = o.tw_q[i];
   const int m = blockIdx.x * nw + warp;
   const int j = blockIdx.y;
   const int kind = blockIdx.z;
@@ -170,22 +185,18 @@ fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict_
   const double nr = o.coll[4 * mm + 2], nz = o.coll[4 * mm + 3];
   const double dr = rho - rs, dz = z - zs;
   const double base = dr * dr + dz * dz, fourrr = 4.0 * rho * rs;
-  // sub-grid of the pair (nodes l = 0, sg, 2 sg, ..; sg divides q/2): the other
-  // nodes are zero and the weight is sg / (4 pi q), i.e. the (q/sg)-node rule
-  const int sg = o.fill_sig[((size_t)(ext ? 1 : 0) * o.M + mm) * o.N + j];
+  const int sg = o.fill_sig[((size_t)(ext ? 1 : 0) * o.M + mm) * o.N + j], c = sg >> 1;   // strides 1, 2, 4
+  const int qs = q / sg, half = qs / 2;
   const double wq = kInv4Pi * sg / q;
   // n . (x - y_l) = (n_r rho + n_z dz) - n_r rho' cos(phi_l), with sg/(4 pi q) folded in
   const double an = (nr * rho + nz * dz) * wq, bn = nr * rs * wq;
-  if (sg > 1)
-    for (int l = lane; l < q; l += 32)
-      if (l % sg) seq[l] = make_double2(0.0, 0.0);
-  for (int i = lane; i * sg <= half; i += 32) {
+  for (int i = lane; i <= half; i += 32) {
     const int l = i * sg;
     const double R2 = fma(fourrr, o.tab_s2[l], base);
     const double inv = rsqrt(R2);
     const double R = R2 * inv, kR = k * R;
     double sn, cs;
-    trig::sincos_ring_tab(kR, o.tab_ring, &sn, &cs);   // table in global memory (L1-resident)
+    fill_sincos(kR, &sn, &cs);
     double2 s;
     if (!deriv) {
       const double iw = inv * wq;
@@ -194,14 +205,15 @@ fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict_
       const double f = fma(-bn, o.tab_cos[l], an) * (inv * inv * inv);
       s = make_double2(f * fma(-kR, sn, -cs), f * fma(kR, cs, -sn));
     }
-    seq[l] = s;
-    if (l > 0 && l < half) seq[q - l] = s;
+    seq[i] = s;
+    if (i > 0 && i < half) seq[qs - i] = s;
   }
-  __syncthreads();                                          // tables and sequences ready
+  __syncthreads();                                          // table and sequences ready
   // With fft_sum_last_q the last stage is not run: each needed mode is the
   // sum of its last-stage block (twiddle 1, output 0).
-  const int rl = o.fft_sum_last_q ? o.fft_rad_q[o.fft_nst_q - 1] : 1;
-  fft::warp_fft(seq, q, tw, o.fft_rad_q, o.fft_nst_q - (rl > 1 ? 1 : 0), lane);
+  const int rl = o.fft_sum_last_q[c] ? o.fft_rad_q[c][o.fft_nst_q[c] - 1] : 1;
+  fft::warp_fft(seq, qs, tw, o.fft_rad_q[c], o.fft_nst_q[c] - (rl > 1 ? 1 : 0), lane, sg);
+  const int *perm = o.fft_perm_q[c];
   if (m >= o.M) return;
   int row = m, col = j;
   double sign = 1.0;
@@ -229,11 +241,11 @@ fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict_
 cudaError_t launch_fill(const ObsDev *d_obs, const ObsDev &h, int oi, double2 *out, int ld_rows,
                         int ld_cols, cudaStream_t st, int chunk_mb) {
   // split-precision plans: samples in FP64, the transform on tensor cores
-  if (h.slices > 0 && h.fill_cdig != nullptr)
+  if (h.slices > 0 && h.fill_list != nullptr)
     return launch_fill_mma(d_obs, h, oi, out, ld_rows, ld_cols, chunk_mb, st);
-  if (h.fft_nst_q > 0) {
+  if (h.fft_nst_q[0] > 0) {                               // then q / 2 and q / 4 have radices too
     const int nw = h.q <= 512 ? 8 : 4;                      // pairs (warps) per CTA
-    const size_t smem = sizeof(double2) * (h.q + (h.q + 1) / 2 + (size_t)nw * h.q);
+    const size_t smem = sizeof(double2) * (h.q + (size_t)nw * h.q);
     static size_t granted = 0;
     cudaError_t e = ensure_dynamic_smem(fill_fft_kernel, smem, granted);
     if (e != cudaSuccess) return e;

@@ -7,7 +7,12 @@
 // Pairing l with h - l (cos(pi n (h - l)/h) = (-1)^n cos(pi n l/h)) folds it to
 //   A_n = sum_{l<L} w_l cos(pi n l / h) u_l,   u = e (n even), o (n odd),
 //   e_l = g_l + g_{h-l},  o_l = g_l - g_{h-l}  (l < h/2),  e_{h/2} = g_{h/2},
-// w_0 = 1, w_l = 2 otherwise; L = h/2 + 1 (h even) or (h + 1)/2 (h odd).
+// w_0 = 1, w_l = 2 otherwise; L = h/2 + 1 (h even) or (h + 1)/2 (h odd). A pair
+// sampled on every sg-th node (axi_fill_subgrid) is the same with h / sg in
+// place of h, so the pairs are taken by stride: the digits and the contraction
+// of the cup's 91% of pairs with q/4 nodes shrink to a quarter. Fill of the cup
+// (432 x 360 pairs, q = 1000): 3.30 ms with every pair on all nodes, zeros
+// between its own, 2.00 ms now.
 // That is two real GEMMs per plan: [cos table of the even modes] x [e of every
 // pair, real and imaginary part as separate columns], likewise odd/o.
 //
@@ -67,15 +72,25 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
   return v;
 }
 
+// One launch of the samples or the transform: pairs list[pair0 .. + npairs) of
+// a proxy set (kinds kind0 .. + nk) and stride class c.
+struct FillPart {
+  int c, pair0, npairs, kind0, nk, turns;   // turns: pairs a warp of the samples takes one after another
+  const int *list;
+};
+
 // Sample kernel. gdig: [2 parts][cols2][kFS][Lp] BF16 bit patterns, read as
 // 32-bit words (two k per word); gex: [2 parts][cols2] exponents (one bit of
-// headroom, as split2_fast wants). Column c2 = 2 (pair_local * kinds + kind)
-// + (0 re, 1 im).
+// headroom, as split2_fast wants). Column c2 = 2 (pair_local * nk + kind - kind0)
+// + (0 re, 1 im). The class's nodes l = i << c, i <= h, carry the whole pair (a
+// pair of a coarser stride that joined the class has zeros between), so a pair
+// sampled on q/4 nodes costs a quarter of the digits and of the contraction.
 __global__ void __launch_bounds__(256, 5)
-fill_samples_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int npairs, int kinds,
-                    uint32_t *__restrict__ gdig, int *__restrict__ gex) {
+fill_samples_kernel(const ObsDev *__restrict__ obs_arr, int oi, FillPart fp, uint32_t *__restrict__ gdig,
+                    int *__restrict__ gex) {
   const ObsDev &o = obs_arr[oi];
-  const int q = o.q, h = q / 2, L = o.fill_L, Lp = o.fill_Lp;
+  const int q = o.q, h = (q / 2) >> fp.c, L = o.fill_L[fp.c], Lp = o.fill_Lp[fp.c];
+  const int npairs = fp.npairs, kinds = fp.nk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   extern __shared__ double2 fseq[];
   longlong2 *ring = reinterpret_cast<longlong2 *>(fseq);   // [1024] (cos, sin) 2^62
@@ -83,116 +98,118 @@ fill_samples_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int n
     ring[i] = make_longlong2(g_ring_q62[i][0], g_ring_q62[i][1]);
   __syncthreads();
   double2 *seq = fseq + trig::kRingTab + (size_t)warp * (h + 1);
-  const int pl = blockIdx.x * kFWarpsA + warp;
-  if (pl >= npairs) return;                       // whole warp; no block barriers below
-  const int kind = blockIdx.y;
-  const int p = pair0 + pl;
-  const int m = p / o.N, j = p % o.N;
+  const int kk = blockIdx.y, kind = fp.kind0 + kk;
   const bool deriv = (o.bc == AXI_BC_NEUMANN) ? true : (kind & 1);
   const bool ext = (o.bc == AXI_BC_TRANSMISSION) && kind >= 2;
   const double k = ext ? o.km : o.k;
   const double *Sp = ext ? o.srcx : o.src;
-  const double rs = Sp[2 * j], zs = Sp[2 * j + 1];
-  const double rho = o.coll[4 * m], z = o.coll[4 * m + 1];
-  const double nr = o.coll[4 * m + 2], nz = o.coll[4 * m + 3];
-  const double dr = rho - rs, dz = z - zs;
-  const double base = dr * dr + dz * dz, fourrr = 4.0 * rho * rs;
-  // sub-grid: nodes l = 0, sg, 2 sg, .. (sg divides h), weight sg / (4 pi q);
-  // the other nodes stay zero, so the transform below is the (q/sg)-node rule
-  const int sg = o.fill_sig[((size_t)(ext ? 1 : 0) * o.M + m) * o.N + j];
-  const double wq = kInv4Pi * sg / q;
-  // n . (x - y_l) = (n_r rho + n_z dz) - n_r rho' cos(phi_l), with sg/(4 pi q) folded in
-  const double an = (nr * rho + nz * dz) * wq, bn = nr * rs * wq;
-  if (sg > 1)
-    for (int l = lane; l <= h; l += 32)
-      if (l % sg) seq[l] = make_double2(0.0, 0.0);
-  for (int i = lane; i * sg <= h; i += 32) {
-    const int l = i * sg;
-    const double R2 = fma(fourrr, o.tab_s2[l], base);
-    const double inv = rsqrt(R2);
-    const double R = R2 * inv, kR = k * R;
-    double sn, cs;
-    trig::sincos_ring_q(kR, ring, &sn, &cs);
-    double2 s;
-    if (!deriv) {
-      const double iw = inv * wq;
-      s = make_double2(cs * iw, sn * iw);
-    } else {
-      const double f = fma(-bn, o.tab_cos[l], an) * (inv * inv * inv);
-      s = make_double2(f * fma(-kR, sn, -cs), f * fma(kR, cs, -sn));
+  for (int turn = 0; turn < fp.turns; ++turn) {
+    const int pl = (blockIdx.x * fp.turns + turn) * kFWarpsA + warp;
+    if (pl >= npairs) return;                       // whole warp; no block barriers below
+    __syncwarp();
+    const int p = fp.list[fp.pair0 + pl];
+    const int m = p / o.N, j = p % o.N;
+    const double rs = Sp[2 * j], zs = Sp[2 * j + 1];
+    const double rho = o.coll[4 * m], z = o.coll[4 * m + 1];
+    const double nr = o.coll[4 * m + 2], nz = o.coll[4 * m + 3];
+    const double dr = rho - rs, dz = z - zs;
+    const double base = dr * dr + dz * dz, fourrr = 4.0 * rho * rs;
+    // the pair's own stride sg (weight sg / (4 pi q)) in units of the class's nodes
+    const int sg = o.fill_sig[((size_t)(ext ? 1 : 0) * o.M + m) * o.N + j], st = sg >> fp.c;
+    const double wq = kInv4Pi * sg / q;
+    // n . (x - y_l) = (n_r rho + n_z dz) - n_r rho' cos(phi_l), with sg/(4 pi q) folded in
+    const double an = (nr * rho + nz * dz) * wq, bn = nr * rs * wq;
+    if (st > 1)
+      for (int l = lane; l <= h; l += 32)
+        if (l % st) seq[l] = make_double2(0.0, 0.0);
+    for (int i = lane; i * st <= h; i += 32) {
+      const int l = i * sg;
+      const double R2 = fma(fourrr, o.tab_s2[l], base);
+      const double inv = rsqrt(R2);
+      const double R = R2 * inv, kR = k * R;
+      double sn, cs;
+      trig::sincos_ring_q(kR, ring, &sn, &cs);
+      double2 s;
+      if (!deriv) {
+        const double iw = inv * wq;
+        s = make_double2(cs * iw, sn * iw);
+      } else {
+        const double f = fma(-bn, o.tab_cos[l], an) * (inv * inv * inv);
+        s = make_double2(f * fma(-kR, sn, -cs), f * fma(kR, cs, -sn));
+      }
+      seq[i * st] = s;
     }
-    seq[l] = s;
-  }
-  __syncwarp();
-  // fold in place: e_l at l, o_l at h - l (l < h/2); the middle e_{h/2} stays
-  const bool mid = (h & 1) == 0;
-  for (int l = lane; l < L; l += 32) {
-    if (mid && l == h / 2) continue;
-    const double2 a = seq[l], b = seq[h - l];
-    seq[l] = make_double2(a.x + b.x, a.y + b.y);
-    seq[h - l] = make_double2(a.x - b.x, a.y - b.y);
-  }
-  __syncwarp();
-  auto eval = [&](int l) { return l < L ? seq[l] : make_double2(0.0, 0.0); };
-  auto oval = [&](int l) {
-    return (l < L && !(mid && l == h / 2)) ? seq[h - l] : make_double2(0.0, 0.0);
-  };
-  unsigned long long ke_r = 0, ke_i = 0, ko_r = 0, ko_i = 0;
-  for (int l = lane; l < L; l += 32) {
-    const double2 e = eval(l), od = oval(l);
-    ke_r = max(ke_r, oz::abs_key(e.x));
-    ke_i = max(ke_i, oz::abs_key(e.y));
-    ko_r = max(ko_r, oz::abs_key(od.x));
-    ko_i = max(ko_i, oz::abs_key(od.y));
-  }
-  ke_r = warp_max_u64(ke_r);
-  ke_i = warp_max_u64(ke_i);
-  ko_r = warp_max_u64(ko_r);
-  ko_i = warp_max_u64(ko_i);
-  const int xe_r = oz::key_exponent(ke_r) + 1, xe_i = oz::key_exponent(ke_i) + 1;
-  const int xo_r = oz::key_exponent(ko_r) + 1, xo_i = oz::key_exponent(ko_i) + 1;
-  const size_t cols2 = (size_t)npairs * kinds * 2;
-  const size_t c2 = 2 * ((size_t)pl * kinds + kind);
-  if (lane == 0) {
-    gex[c2] = xe_r;
-    gex[c2 + 1] = xe_i;
-    gex[cols2 + c2] = xo_r;
-    gex[cols2 + c2 + 1] = xo_i;
-  }
-  const int wpr = Lp / 2;                                  // words per digit row
-  if (!o.fill_tc) {
-    // [part][cols2][kFS][Lp]
-    uint32_t *de_r = gdig + (c2 * kFS) * wpr;
-    uint32_t *de_i = gdig + ((c2 + 1) * kFS) * wpr;
-    uint32_t *do_r = gdig + ((cols2 + c2) * kFS) * wpr;
-    uint32_t *do_i = gdig + ((cols2 + c2 + 1) * kFS) * wpr;
-    for (int w = lane; w < wpr; w += 32) {
-      const double2 e0 = eval(2 * w), e1 = eval(2 * w + 1);
-      const double2 o0 = oval(2 * w), o1 = oval(2 * w + 1);
-      oz::split2_fast<kFS>(e0.x, e1.x, xe_r, de_r + w, wpr);
-      oz::split2_fast<kFS>(e0.y, e1.y, xe_i, de_i + w, wpr);
-      oz::split2_fast<kFS>(o0.x, o1.x, xo_r, do_r + w, wpr);
-      oz::split2_fast<kFS>(o0.y, o1.y, xo_i, do_i + w, wpr);
+    __syncwarp();
+    // fold in place: e_l at l, o_l at h - l (l < h/2); the middle e_{h/2} stays
+    const bool mid = (h & 1) == 0;
+    for (int l = lane; l < L; l += 32) {
+      if (mid && l == h / 2) continue;
+      const double2 a = seq[l], b = seq[h - l];
+      seq[l] = make_double2(a.x + b.x, a.y + b.y);
+      seq[h - l] = make_double2(a.x - b.x, a.y - b.y);
     }
-  } else {
-    // tcgen05 tiles: [part][128-column block][16-k chunk][digit] K-major
-    // no-swizzle tiles of 128 rows x 16 k (4096 bytes, 1024 words); column c
-    // is row c mod 128, word w holds k = 2w, 2w + 1
-    const int nch = Lp / 16, nblk = ((int)cols2 + 127) / 128;
-    auto tile = [&](int pt, size_t c) {
-      const int cb = (int)(c >> 7), r = (int)(c & 127);
-      return gdig + ((size_t)(pt * nblk + cb) * nch) * kFS * 1024 + (r >> 3) * 64 + (r & 7) * 4;
+    __syncwarp();
+    auto eval = [&](int l) { return l < L ? seq[l] : make_double2(0.0, 0.0); };
+    auto oval = [&](int l) {
+      return (l < L && !(mid && l == h / 2)) ? seq[h - l] : make_double2(0.0, 0.0);
     };
-    uint32_t *de_r = tile(0, c2), *de_i = tile(0, c2 + 1);
-    uint32_t *do_r = tile(1, c2), *do_i = tile(1, c2 + 1);
-    for (int w = lane; w < wpr; w += 32) {
-      const double2 e0 = eval(2 * w), e1 = eval(2 * w + 1);
-      const double2 o0 = oval(2 * w), o1 = oval(2 * w + 1);
-      const size_t off = (size_t)(w >> 3) * kFS * 1024 + ((w & 7) >> 2) * 32 + (w & 3);
-      oz::split2_fast<kFS>(e0.x, e1.x, xe_r, de_r + off, 1024);
-      oz::split2_fast<kFS>(e0.y, e1.y, xe_i, de_i + off, 1024);
-      oz::split2_fast<kFS>(o0.x, o1.x, xo_r, do_r + off, 1024);
-      oz::split2_fast<kFS>(o0.y, o1.y, xo_i, do_i + off, 1024);
+    unsigned long long ke_r = 0, ke_i = 0, ko_r = 0, ko_i = 0;
+    for (int l = lane; l < L; l += 32) {
+      const double2 e = eval(l), od = oval(l);
+      ke_r = max(ke_r, oz::abs_key(e.x));
+      ke_i = max(ke_i, oz::abs_key(e.y));
+      ko_r = max(ko_r, oz::abs_key(od.x));
+      ko_i = max(ko_i, oz::abs_key(od.y));
+    }
+    ke_r = warp_max_u64(ke_r);
+    ke_i = warp_max_u64(ke_i);
+    ko_r = warp_max_u64(ko_r);
+    ko_i = warp_max_u64(ko_i);
+    const int xe_r = oz::key_exponent(ke_r) + 1, xe_i = oz::key_exponent(ke_i) + 1;
+    const int xo_r = oz::key_exponent(ko_r) + 1, xo_i = oz::key_exponent(ko_i) + 1;
+    const size_t cols2 = (size_t)npairs * kinds * 2;
+    const size_t c2 = 2 * ((size_t)pl * kinds + kk);
+    if (lane == 0) {
+      gex[c2] = xe_r;
+      gex[c2 + 1] = xe_i;
+      gex[cols2 + c2] = xo_r;
+      gex[cols2 + c2 + 1] = xo_i;
+    }
+    const int wpr = Lp / 2;                                  // words per digit row
+    if (!o.fill_tc[fp.c]) {
+      // [part][cols2][kFS][Lp]
+      uint32_t *de_r = gdig + (c2 * kFS) * wpr;
+      uint32_t *de_i = gdig + ((c2 + 1) * kFS) * wpr;
+      uint32_t *do_r = gdig + ((cols2 + c2) * kFS) * wpr;
+      uint32_t *do_i = gdig + ((cols2 + c2 + 1) * kFS) * wpr;
+      for (int w = lane; w < wpr; w += 32) {
+        const double2 e0 = eval(2 * w), e1 = eval(2 * w + 1);
+        const double2 o0 = oval(2 * w), o1 = oval(2 * w + 1);
+        oz::split2_fast<kFS>(e0.x, e1.x, xe_r, de_r + w, wpr);
+        oz::split2_fast<kFS>(e0.y, e1.y, xe_i, de_i + w, wpr);
+        oz::split2_fast<kFS>(o0.x, o1.x, xo_r, do_r + w, wpr);
+        oz::split2_fast<kFS>(o0.y, o1.y, xo_i, do_i + w, wpr);
+      }
+    } else {
+      // tcgen05 tiles: [part][128-column block][16-k chunk][digit] K-major
+      // no-swizzle tiles of 128 rows x 16 k (4096 bytes, 1024 words); column c
+      // is row c mod 128, word w holds k = 2w, 2w + 1
+      const int nch = Lp / 16, nblk = ((int)cols2 + 127) / 128;
+      auto tile = [&](int pt, size_t c) {
+        const int cb = (int)(c >> 7), r = (int)(c & 127);
+        return gdig + ((size_t)(pt * nblk + cb) * nch) * kFS * 1024 + (r >> 3) * 64 + (r & 7) * 4;
+      };
+      uint32_t *de_r = tile(0, c2), *de_i = tile(0, c2 + 1);
+      uint32_t *do_r = tile(1, c2), *do_i = tile(1, c2 + 1);
+      for (int w = lane; w < wpr; w += 32) {
+        const double2 e0 = eval(2 * w), e1 = eval(2 * w + 1);
+        const double2 o0 = oval(2 * w), o1 = oval(2 * w + 1);
+        const size_t off = (size_t)(w >> 3) * kFS * 1024 + ((w & 7) >> 2) * 32 + (w & 3);
+        oz::split2_fast<kFS>(e0.x, e1.x, xe_r, de_r + off, 1024);
+        oz::split2_fast<kFS>(e0.y, e1.y, xe_i, de_i + off, 1024);
+        oz::split2_fast<kFS>(o0.x, o1.x, xo_r, do_r + off, 1024);
+        oz::split2_fast<kFS>(o0.y, o1.y, xo_i, do_i + off, 1024);
+      }
     }
   }
 }
@@ -201,11 +218,13 @@ fill_samples_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int n
 // n = 2 r' + part, rows with n >= D are zero). Columns: NT real columns per
 // CTA. Warp w < MT * NT / 8 computes the 16 x 8 tile (w / (NT/8), w % (NT/8)).
 __global__ void __launch_bounds__(kFThreadsB)
-fill_gemm_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int npairs, int kinds,
+fill_gemm_kernel(const ObsDev *__restrict__ obs_arr, int oi, FillPart fp,
                  int NT, const uint32_t *__restrict__ gdig, const int *__restrict__ gex,
                  double2 *__restrict__ out, int ld_rows, int ld_cols) {
   const ObsDev &o = obs_arr[oi];
-  const int Lp = o.fill_Lp, MR = o.fill_MR, D = o.D;
+  const int npairs = fp.npairs, kinds = fp.nk;
+  const unsigned short *cdig = o.fill_cdig[fp.c];
+  const int Lp = o.fill_Lp[fp.c], MR = o.fill_MR, D = o.D;
   const int rows = 2 * MR, MT = rows / 16, nt8 = NT / 8;
   const int cols2 = npairs * kinds * 2;
   const int c0 = blockIdx.x * NT;
@@ -238,7 +257,7 @@ fill_gemm_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int npai
     for (int e = tid; e < rows * kFS * 4; e += kFThreadsB) {
       const int u = e & 3, sr = e >> 2;                     // sr = s * rows + row
       oz::cp_async16(cs + (size_t)sr * kFLD + 8 * u,
-                     o.fill_cdig + (size_t)sr * Lp + ch * kFKC + 8 * u, true);
+                     cdig + (size_t)sr * Lp + ch * kFKC + 8 * u, true);
     }
     for (int e = tid; e < 2 * NT * kFS * 4; e += kFThreadsB) {
       const int u = e & 3, r = e >> 2;                      // r = (pt * kFS + s) * NT + c
@@ -320,8 +339,8 @@ fill_gemm_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int npai
       const int E = ce + gex[(size_t)part * cols2 + colc + c];
       vv[c] = oz::scaled_to_double(hi[e], E - 28) + oz::scaled_to_double(lo[e], E - 7 * (kFS + 1));
     }
-    const int cp = colc / 2, kind = cp % kinds, pl = cp / kinds;
-    const int p = pair0 + pl, m = p / o.N, j = p % o.N;
+    const int cp = colc / 2, kind = fp.kind0 + cp % kinds, pl = cp / kinds;
+    const int p = fp.list[fp.pair0 + pl], m = p / o.N, j = p % o.N;
     int orow = m, ocol = j;
     double sign = 1.0;
     if (o.bc == AXI_BC_TRANSMISSION) {
@@ -379,11 +398,12 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
 
 template <int kTcStages, int kTcAcc>
 __global__ void __launch_bounds__(kTcThreads, 1)
-fill_gemm_tc_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int npairs, int kinds,
+fill_gemm_tc_kernel(const ObsDev *__restrict__ obs_arr, int oi, FillPart fp,
                     const uint32_t *__restrict__ gdig, const int *__restrict__ gex,
                     double2 *__restrict__ out, int ld_rows, int ld_cols) {
   const ObsDev &o = obs_arr[oi];
-  const int Lp = o.fill_Lp, MR = o.fill_MR, D = o.D;
+  const int npairs = fp.npairs, kinds = fp.nk;
+  const int Lp = o.fill_Lp[fp.c], MR = o.fill_MR, D = o.D;
   const int cols2 = npairs * kinds * 2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nch = Lp / 16, nblk = (cols2 + kTcCols - 1) / kTcCols;
@@ -430,7 +450,7 @@ fill_gemm_tc_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int n
       unsigned char *buf = tsm + (size_t)b * stage_bytes;
       const unsigned char *ga = reinterpret_cast<const unsigned char *>(gdig) +
                                 ((size_t)(part * nblk + cb) * nch + ch) * a_bytes;
-      const unsigned char *gb = reinterpret_cast<const unsigned char *>(o.fill_cdig) +
+      const unsigned char *gb = reinterpret_cast<const unsigned char *>(o.fill_cdig[fp.c]) +
                                 ((size_t)part * nch + ch) * b_bytes;
       tc::mbar_arrive_expect_tx(&full[b], a_bytes + b_bytes);
       tc::bulk_g2s(buf, ga, a_bytes, &full[b]);
@@ -502,8 +522,8 @@ fill_gemm_tc_kernel(const ObsDev *__restrict__ obs_arr, int oi, int pair0, int n
       tile_of(i, part, cb);
       const int col = cb * kTcCols + lb + lane;
       const int ex_col = col < cols2 ? gex[(size_t)part * cols2 + col] : 0;
-      const int cp = col / 2, kind = cp % kinds, pl = cp / kinds;
-      const int p = pair0 + pl, m = p / o.N, j = p % o.N;
+      const int cp = col / 2, kind = fp.kind0 + cp % kinds, pl = cp / kinds;
+      const int p = col < cols2 ? fp.list[fp.pair0 + pl] : 0, m = p / o.N, j = p % o.N;
       int orow = m, ocol = j;
       double sign = 1.0;
       if (o.bc == AXI_BC_TRANSMISSION) {
@@ -579,51 +599,65 @@ size_t fill_gemm_smem(int MR) {
 
 cudaError_t launch_fill_mma(const ObsDev *d_obs, const ObsDev &h, int oi, double2 *out,
                             int ld_rows, int ld_cols, int chunk_mb, cudaStream_t st) {
-  const int kinds = h.bc == AXI_BC_TRANSMISSION ? 4 : 1;
-  const int npairs_total = h.M * h.N;
-  // ring pairs per chunk: the plan's (its scratch holds that many), or fewer
-  // so that one chunk's sample digits stay in L2 between the two kernels
-  int chunk = h.fill_chunk_pairs;
-  if (chunk_mb > 0) {
-    const size_t per_pair = (size_t)2 * 2 * kinds * kFillDigits * h.fill_Lp * sizeof(unsigned short);
-    const size_t want = ((size_t)chunk_mb << 20) / per_pair;
-    chunk = (int)std::max<size_t>(8, std::min<size_t>((size_t)chunk, want));
-  }
+  const bool trans = h.bc == AXI_BC_TRANSMISSION;
   const int NT = fill_gemm_cols(h.fill_MR);
-  const size_t smemA = sizeof(double2) * ((size_t)trig::kRingTab + (size_t)kFWarpsA * (h.q / 2 + 1));
-  const bool tc = h.fill_tc != 0;
-  // one CTA per SM, 4 stages; two accumulator sets when 16 MR TMEM columns fit
-  const bool two = h.fill_MR <= 32;
-  const size_t smemB = tc ? (size_t)4 * tc_stage_bytes(h.fill_MR) : fill_gemm_smem(h.fill_MR);
   static size_t grantedA = 0, grantedB = 0, grantedT2 = 0, grantedT1 = 0;
-  cudaError_t e = ensure_dynamic_smem(fill_samples_kernel, smemA, grantedA);
-  if (e != cudaSuccess) return e;
-  e = !tc ? ensure_dynamic_smem(fill_gemm_kernel, smemB, grantedB)
-          : two ? ensure_dynamic_smem(fill_gemm_tc_kernel<4, 2>, smemB, grantedT2)
-                : ensure_dynamic_smem(fill_gemm_tc_kernel<4, 1>, smemB, grantedT1);
-  if (e != cudaSuccess) return e;
-  for (int pair0 = 0; pair0 < npairs_total; pair0 += chunk) {
-    const int np = min(chunk, npairs_total - pair0);
-    fill_samples_kernel<<<dim3((np + kFWarpsA - 1) / kFWarpsA, kinds), 32 * kFWarpsA, smemA, st>>>(
-        d_obs, oi, pair0, np, kinds, h.fill_gdig, h.fill_gex);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int cols2 = np * kinds * 2;
-    // persistent: one CTA per SM
-    const int ntiles = 2 * ((cols2 + kTcCols - 1) / kTcCols);
-    const dim3 tgrid(min(ntiles, sm_count()));
-    if (tc && two)
-      fill_gemm_tc_kernel<4, 2><<<tgrid, kTcThreads, smemB, st>>>(
-          d_obs, oi, pair0, np, kinds, h.fill_gdig, h.fill_gex, out, ld_rows, ld_cols);
-    else if (tc)
-      fill_gemm_tc_kernel<4, 1><<<tgrid, kTcThreads, smemB, st>>>(
-          d_obs, oi, pair0, np, kinds, h.fill_gdig, h.fill_gex, out, ld_rows, ld_cols);
-    else
-      fill_gemm_kernel<<<(cols2 + NT - 1) / NT, kFThreadsB, smemB, st>>>(
-          d_obs, oi, pair0, np, kinds, NT, h.fill_gdig, h.fill_gex, out, ld_rows, ld_cols);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  for (int set = 0; set < (trans ? 2 : 1); ++set)
+    for (int c = 0; c < 3; ++c) {
+      const int total = h.fill_cnt[set][c];
+      if (total == 0) continue;
+      FillPart fp;
+      fp.c = c;
+      fp.kind0 = trans ? 2 * set : 0;
+      fp.nk = trans ? 2 : 1;
+      fp.list = h.fill_list + h.fill_off[set][c];
+      // ring pairs per chunk: what the scratch holds, or fewer so that one
+      // chunk's sample digits stay in L2 between the two kernels
+      const size_t per_pair = fill_pair_bytes(h, c);
+      size_t chunk = (h.fill_cap - fill_pad_bytes(h, c)) / per_pair;
+      if (chunk_mb > 0) chunk = std::max<size_t>(8, std::min<size_t>(chunk, ((size_t)chunk_mb << 20) / per_pair));
+      const size_t smemA =
+          sizeof(double2) * ((size_t)trig::kRingTab + (size_t)kFWarpsA * (((h.q / 2) >> c) + 1));
+      const bool tc = h.fill_tc[c] != 0;
+      // one CTA per SM, 4 stages; two accumulator sets when 16 MR TMEM columns fit
+      const bool two = h.fill_MR <= 32;
+      const size_t smemB = tc ? (size_t)4 * tc_stage_bytes(h.fill_MR) : fill_gemm_smem(h.fill_MR);
+      cudaError_t e = ensure_dynamic_smem(fill_samples_kernel, smemA, grantedA);
+      if (e != cudaSuccess) return e;
+      e = !tc ? ensure_dynamic_smem(fill_gemm_kernel, smemB, grantedB)
+              : two ? ensure_dynamic_smem(fill_gemm_tc_kernel<4, 2>, smemB, grantedT2)
+                    : ensure_dynamic_smem(fill_gemm_tc_kernel<4, 1>, smemB, grantedT1);
+      if (e != cudaSuccess) return e;
+      for (int pair0 = 0; pair0 < total; pair0 += (int)chunk) {
+        const int np = (int)std::min<size_t>(chunk, total - pair0);
+        fp.pair0 = pair0;
+        fp.npairs = np;
+        // several pairs a warp share a CTA's copy of the sin/cos table, while eight
+        // waves of CTAs (five an SM) are left to even out the tail
+        const int waves = np * fp.nk / (kFWarpsA * 5 * sm_count());
+        fp.turns = std::max(1, std::min(4, waves / 8));
+        const int per_cta = kFWarpsA * fp.turns;
+        fill_samples_kernel<<<dim3((np + per_cta - 1) / per_cta, fp.nk), 32 * kFWarpsA, smemA, st>>>(
+            d_obs, oi, fp, h.fill_gdig, h.fill_gex);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        const int cols2 = np * fp.nk * 2;
+        // persistent: one CTA per SM
+        const int ntiles = 2 * ((cols2 + kTcCols - 1) / kTcCols);
+        const dim3 tgrid(min(ntiles, sm_count()));
+        if (tc && two)
+          fill_gemm_tc_kernel<4, 2><<<tgrid, kTcThreads, smemB, st>>>(d_obs, oi, fp, h.fill_gdig, h.fill_gex, out,
+                                                                    ld_rows, ld_cols);
+        else if (tc)
+          fill_gemm_tc_kernel<4, 1><<<tgrid, kTcThreads, smemB, st>>>(d_obs, oi, fp, h.fill_gdig, h.fill_gex, out,
+                                                                    ld_rows, ld_cols);
+        else
+          fill_gemm_kernel<<<(cols2 + NT - 1) / NT, kFThreadsB, smemB, st>>>(d_obs, oi, fp, NT, h.fill_gdig,
+                                                                           h.fill_gex, out, ld_rows, ld_cols);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+      }
+    }
   return cudaSuccess;
 }
 
