@@ -516,6 +516,8 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
     d.npanels = (d.cols + axi::kNB - 1) / axi::kNB;
     d.slices = slices;
     d.k = o.k; d.km = o.bc == AXI_BC_TRANSMISSION ? o.k_minus : 0.0;
+    d.ph = axi::trig::ring_phase(o.k);
+    if (o.bc == AXI_BC_TRANSMISSION) d.phm = axi::trig::ring_phase(o.k_minus);
     h.coll.assign(o.h_coll, o.h_coll + 4 * o.M);
     h.src.assign(o.h_src, o.h_src + 2 * o.N);
     if (o.bc == AXI_BC_TRANSMISSION) h.srcx.assign(o.h_src_ext, o.h_src_ext + 2 * o.N);

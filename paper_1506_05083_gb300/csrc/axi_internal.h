@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/axi_mfs.h"
+#include "trig.cuh"
 
 namespace axi {
 
@@ -19,12 +20,12 @@ constexpr int kPlanTsvd = 1 << 17;           // AXI_PLAN_TSVD
 // Schedule choices of a plan (axi_plan_set_tuning, axi_operator_autotune).
 struct Tuning {
   int next_update = 0;    // 0 auto, 1 native FP64, 2 split digits (split plans)
-  int panel_cluster = 0;  // 0 auto (by the number of tasks), else 1, 2 or 4 CTAs per mode
+  int panel_cluster = 0;  // 0 auto (by rows and number of tasks), else 1, 2 or 4 CTAs per mode
   int rest_grid = 0;      // split trailing update: 0 auto (2 where the update reads Y^H digits,
                           // else 4), 1 mma.sync persistent (one CTA per SM), 2 tcgen05 kernel,
                           // 3 the same with one CTA per SM (room for a critical-path CTA beside it),
                           // 4 mma.sync, one CTA per (task, column tile)
-  int panel_threads = 0;  // 0 auto (256 on one CTA with more than 128 rows, else 128), 128, 256
+  int panel_threads = 0;  // 0 auto (256 on one CTA with 129 to 288 rows, else 128), 128, 256
   int crit_stream = 0;    // 0 the panel chain on the caller's stream, 1 on a stream of the
                           // operator with the device's highest priority
   int fill_chunk_mb = 0;  // split fill: 0 the plan's chunk (up to 512 MB of sample digits),
@@ -52,6 +53,7 @@ struct ObsDev {
   int npanels;            // ceil(cols / kNB)
   int slices;             // 0: native FP64 updates; 4..8: BF16 digits per FP64 value
   double k, km;           // exterior / interior wavenumber
+  trig::RingPhase ph, phm;  // the same as table steps per unit length (trig.cuh)
   const double *coll;     // [M][4] rho, z, n_rho, n_z
   const double *src;      // [N][2] interior proxies
   const double *srcx;     // [N][2] exterior proxies (transmission) or null

@@ -58,36 +58,32 @@ __device__ const long long g_field_ring_q62[trig::kRingTab][2] = {
 #include "ring_table_q62.inc"
 };
 
-// sin and cos of |x| < 2^20 in fixed point with the table read through L1, any
-// other x (NaN too) by the library.
-__device__ __forceinline__ void sincos_field(double x, double *sn, double *cs) {
-  if (fabs(x) < 1048576.0)
-    trig::sincos_ring_q(x, reinterpret_cast<const longlong2 *>(g_field_ring_q62), sn, cs);
-  else
-    sincos(x, sn, cs);
-}
-
 // Kernel value times 4 pi: e^{ikR}/R, its normal derivative, or e^{-ik x.y}.
 // The FP64 pipe bounds the evaluation (1/64 rate), so the square root comes
 // from rsqrt with one correction (a division and a square root cost twice
-// that), and sin/cos run in fixed point: 21 FP64 operations for the potential.
+// that), and the phase, sin and cos run in fixed point (trig::sincos_phase):
+// 16 FP64 operations for the potential.
 template <int KIND>
-__device__ __forceinline__ double2 field_kernel(double k, double tx, double ty, double tz, double nx, double ny,
-                                                double nz, double yx, double yy, double yz) {
+__device__ __forceinline__ double2 field_kernel(const trig::RingPhase &ph, double tx, double ty, double tz, double nx,
+                                                double ny, double nz, double yx, double yy, double yz) {
+  const longlong2 *tab = reinterpret_cast<const longlong2 *>(g_field_ring_q62);   // through L1
+  const trig::PhaseOffset none{0, 0};
   double sn, cs;
-  if (KIND == AXI_EVAL_FAR_FIELD) {                        // (tx, ty, tz) = -k x
-    sincos_field(fma(tx, yx, fma(ty, yy, tz * yz)), &sn, &cs);
-    return make_double2(cs, sn);
+  if (KIND == AXI_EVAL_FAR_FIELD) {
+    const double a = fma(tx, yx, fma(ty, yy, tz * yz));
+    trig::sincos_phase(fabs(a), ph, none, tab, &sn, &cs);
+    // -sin(k a) = -sign(a) sin(k |a|), on the bits
+    return make_double2(cs, __longlong_as_double(__double_as_longlong(sn) ^
+                                                 (~__double_as_longlong(a) & (long long)(1ull << 63))));
   }
   const double dx = tx - yx, dy = ty - yy, dz = tz - yz;
   const double R2 = fma(dx, dx, fma(dy, dy, dz * dz));
   const double inv = rsqrt(R2);
   double R = R2 * inv;
   R = fma(0.5 * inv, fma(-R, R, R2), R);                   // to half a unit in the last place
-  const double kR = k * R;
-  sincos_field(kR, &sn, &cs);
+  trig::sincos_phase(R, ph, none, tab, &sn, &cs);
   if (KIND == AXI_EVAL_POTENTIAL) return make_double2(cs * inv, sn * inv);
-  const double f = fma(nx, dx, fma(ny, dy, nz * dz)) * (inv * inv) * inv;
+  const double f = fma(nx, dx, fma(ny, dy, nz * dz)) * (inv * inv) * inv, kR = ph.k * R;
   return make_double2(f * fma(-kR, sn, -cs), f * fma(kR, cs, -sn));   // (ikR - 1) e^{ikR}
 }
 
@@ -98,7 +94,7 @@ __device__ __forceinline__ double2 field_kernel(double k, double tx, double ty, 
 // group's waves, NW chosen to fit them (a fixed group of 8 spent 32 FP64
 // operations a value on phases and sums of waves that were not there: the
 // potential at 4096 targets of 21600 sources, 4 waves, took 12.9 ms and now takes
-// 6.2). The partial sums of a cluster are added by its first CTA in rank order.
+// 5.2). The partial sums of a cluster are added by its first CTA in rank order.
 constexpr int kWG = 16;
 template <int KIND, int NW, bool LAT>
 __global__ void __launch_bounds__(kThreads)
@@ -112,9 +108,8 @@ eval_kernel(const ObsDev *__restrict__ od, int W, const double2 *__restrict__ si
   const int w0 = blockIdx.y * NW;
   const int nw = min(NW, W - w0);
   const int P = o.P, cols = o.cols;
-  const double k = o.k;
-  const double ts = KIND == AXI_EVAL_FAR_FIELD ? -k : 1.0;
-  const double tx = ts * targets[3 * t], ty = ts * targets[3 * t + 1], tz = ts * targets[3 * t + 2];
+  const double tx = targets[3 * t], ty = targets[3 * t + 1], tz = targets[3 * t + 2];
+  const trig::RingPhase ph = o.ph;
   double nx = 0, ny = 0, nz = 0;
   if (KIND == AXI_EVAL_NORMAL_DERIV) { nx = normals[3 * t]; ny = normals[3 * t + 1]; nz = normals[3 * t + 2]; }
   __shared__ double2 phase[LAT ? NW : 1][9];
@@ -123,7 +118,7 @@ eval_kernel(const ObsDev *__restrict__ od, int W, const double2 *__restrict__ si
       const int w = e / 9, im = e % 9;
       double sn = 0.0, cs = 0.0;
       if (w < nw)
-        sincos(k * (dirs[3 * (w0 + w)] * (im / 3 - 1) * ex + dirs[3 * (w0 + w) + 1] * (im % 3 - 1) * ey), &sn, &cs);
+        sincos(ph.k * (dirs[3 * (w0 + w)] * (im / 3 - 1) * ex + dirs[3 * (w0 + w) + 1] * (im % 3 - 1) * ey), &sn, &cs);
       phase[w][im] = make_double2(cs, sn);
     }
     __syncthreads();
@@ -144,7 +139,7 @@ eval_kernel(const ObsDev *__restrict__ od, int W, const double2 *__restrict__ si
       for (int w = 0; w < NW; ++w) val[w] = make_double2(0.0, 0.0);
       for (int im = 0; im < 9; ++im) {
         if (im == 4) continue;                             // central copy excluded (A_else)
-        const double2 kv = field_kernel<KIND>(k, tx, ty, tz, nx, ny, nz, yx + (im / 3 - 1) * ex,
+        const double2 kv = field_kernel<KIND>(ph, tx, ty, tz, nx, ny, nz, yx + (im / 3 - 1) * ex,
                                               yy + (im % 3 - 1) * ey, yz);
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
@@ -154,7 +149,7 @@ eval_kernel(const ObsDev *__restrict__ od, int W, const double2 *__restrict__ si
         }
       }
     } else {
-      val[0] = field_kernel<KIND>(k, tx, ty, tz, nx, ny, nz, yx, yy, yz);
+      val[0] = field_kernel<KIND>(ph, tx, ty, tz, nx, ny, nz, yx, yy, yz);
     }
 #pragma unroll
     for (int w = 0; w < NW; ++w) {

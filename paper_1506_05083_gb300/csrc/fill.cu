@@ -144,13 +144,6 @@ __device__ const long long g_fill_ring_q62[trig::kRingTab][2] = {
 #include "ring_table_q62.inc"
 };
 
-__device__ __forceinline__ void fill_sincos(double x, double *sn, double *cs) {
-  if (fabs(x) < 1048576.0)
-    trig::sincos_ring_q(x, reinterpret_cast<const longlong2 *>(g_fill_ring_q62), sn, cs);
-  else
-    sincos(x, sn, cs);
-}
-
 // FFT variant (q = 2^a 3^b 5^c): one warp per (m, j) pair evaluates the samples
 // of its sub-grid (nodes l = 0, sg, 2 sg, .., i.e. the trapezoid rule on qs =
 // q / sg nodes), mirrors them into the full even sequence of length qs and
@@ -160,7 +153,7 @@ __device__ __forceinline__ void fill_sincos(double x, double *sn, double *cs) {
 // FP64 pipe bounds it; sin and cos run in fixed point, and the transform has
 // the pair's own length (with q nodes for every pair, the others zero, and FP64
 // table sincos the transmission body of 134 x 111 pairs, P = 72, took 1.93 ms,
-// now 0.97 ms).
+// now 0.92 ms).
 __global__ void __launch_bounds__(256)
 fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict__ out,
                 int ld_rows, int ld_cols) {
@@ -178,6 +171,7 @@ fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict_
   const bool deriv = (o.bc == AXI_BC_NEUMANN) ? true : (kind & 1);
   const bool ext = (o.bc == AXI_BC_TRANSMISSION) && kind >= 2;
   const double k = ext ? o.km : o.k;
+  const trig::RingPhase ph = ext ? o.phm : o.ph;
   const double *S = ext ? o.srcx : o.src;
   const double rs = S[2 * j], zs = S[2 * j + 1];
   const int mm = m < o.M ? m : o.M - 1;
@@ -196,7 +190,7 @@ fill_fft_kernel(const ObsDev *__restrict__ obs_arr, int oi, double2 *__restrict_
     const double inv = rsqrt(R2);
     const double R = R2 * inv, kR = k * R;
     double sn, cs;
-    fill_sincos(kR, &sn, &cs);
+    trig::sincos_phase(R, ph, trig::PhaseOffset{0, 0}, reinterpret_cast<const longlong2 *>(g_fill_ring_q62), &sn, &cs);
     double2 s;
     if (!deriv) {
       const double iw = inv * wq;

@@ -12,12 +12,12 @@
 // place of h, so the pairs are taken by stride: the digits and the contraction
 // of the cup's 91% of pairs with q/4 nodes shrink to a quarter. Fill of the cup
 // (432 x 360 pairs, q = 1000): 3.30 ms with every pair on all nodes, zeros
-// between its own, 2.00 ms now.
+// between its own, 1.89 ms now.
 // That is two real GEMMs per plan: [cos table of the even modes] x [e of every
 // pair, real and imaginary part as separate columns], likewise odd/o.
 //
 //   fill_samples_kernel  one warp per (pair, kind): FP64 samples (sin/cos of
-//                        k R in 64-bit fixed point, trig::sincos_ring_q), the fold,
+//                        k R in 64-bit fixed point, trig::sincos_phase), the fold,
 //                        per-column exponents and S = 8 balanced digits of
 //                        e and o (split2_fast), written to a scratch buffer;
 //   fill_gemm_tc_kernel  (Lp <= 448, MR <= 64) the same GEMM on the fifth-
@@ -102,6 +102,7 @@ fill_samples_kernel(const ObsDev *__restrict__ obs_arr, int oi, FillPart fp, uin
   const bool deriv = (o.bc == AXI_BC_NEUMANN) ? true : (kind & 1);
   const bool ext = (o.bc == AXI_BC_TRANSMISSION) && kind >= 2;
   const double k = ext ? o.km : o.k;
+  const trig::RingPhase ph = ext ? o.phm : o.ph;
   const double *Sp = ext ? o.srcx : o.src;
   for (int turn = 0; turn < fp.turns; ++turn) {
     const int pl = (blockIdx.x * fp.turns + turn) * kFWarpsA + warp;
@@ -128,7 +129,7 @@ fill_samples_kernel(const ObsDev *__restrict__ obs_arr, int oi, FillPart fp, uin
       const double inv = rsqrt(R2);
       const double R = R2 * inv, kR = k * R;
       double sn, cs;
-      trig::sincos_ring_q(kR, ring, &sn, &cs);
+      trig::sincos_phase(R, ph, trig::PhaseOffset{0, 0}, ring, &sn, &cs);
       double2 s;
       if (!deriv) {
         const double iw = inv * wq;

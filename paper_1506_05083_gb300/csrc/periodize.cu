@@ -446,11 +446,11 @@ q_w_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__re
 // Cartesian derivative of G, each summed over the images with their
 // coefficients (the same for every sample, so the sum and the transform
 // exchange), and two warp FFTs give every mode; the row pair's two rows are
-// written for all P modes (column (n mod P) N + j). The FP64 pipe bounds it: 33
-// operations a sample and image (sin and cos in fixed point, table through
+// written for all P modes (column (n mod P) N + j). The FP64 pipe bounds it: 24
+// operations a sample and image (phase, sin and cos in fixed point, table through
 // L1), and one pair of FFTs a row pair instead of one an image. 2048 x 15570
 // entries, P = 90: 32.6 ms with an FFT pair an image and the library's sincos,
-// now 10.8 ms.
+// now 9.0 ms.
 // ---------------------------------------------------------------------------
 
 constexpr int kCWarps = 4;
@@ -459,15 +459,8 @@ __device__ const long long g_c_ring_q62[trig::kRingTab][2] = {
 #include "ring_table_q62.inc"
 };
 
-__device__ __forceinline__ void c_sincos(double x, double *sn, double *cs) {
-  if (fabs(x) < 1048576.0)
-    trig::sincos_ring_q(x, reinterpret_cast<const longlong2 *>(g_c_ring_q62), sn, cs);
-  else
-    sincos(x, sn, cs);
-}
-
 // Shared memory of c_kernel: twiddles, FFT positions, and per warp the samples
-// of both rows and nine images of (x, y, coefficient).
+// of both rows and nine images of (x, y), phase.
 __host__ __device__ inline size_t c_warp_smem(int P) { return 2 * (size_t)P + 18; }   // in double2
 
 __global__ void __launch_bounds__(32 * kCWarps)
@@ -479,7 +472,7 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
   double2 *tw = c_sh;                                           // [P] e^{-2 pi i r / P}
   int *perm = reinterpret_cast<int *>(c_sh + P);                // [P]
   double2 *sv = c_sh + P + (P + 1) / 2 + (size_t)warp * c_warp_smem(P), *sd = sv + P;
-  double2 *img = sd + P;                                        // [9][2]: point (x, y), coefficient
+  double2 *img = sd + P;                                        // [9][2]: point (x, y), phase of the coefficient
   const bool fft = o.fft_nst > 0;
   for (int i = threadIdx.x; i < P; i += blockDim.x) {
     tw[i] = o.tw_P[i];
@@ -495,6 +488,7 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
   const double ex = cell.ex, ey = cell.ey, hx = 0.5 * ex, hy = 0.5 * ey, z0 = cell.z0;
   const double k = o.k, rs = o.src[2 * j], zs = o.src[2 * j + 1];
   const double wgt = 1.0 / (4.0 * 3.14159265358979323846 * P);
+  const trig::RingPhase ph = o.ph;
   const int axis = grp == 0 ? 0 : grp == 1 ? 1 : 2;
   const int npts = grp < 2 ? 6 : 9;
   const double z = grp == 2 ? z0 : grp == 3 ? -z0 : z0 * gb, dz = z - zs, dz2 = dz * dz;
@@ -529,8 +523,8 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
       y = hy * gb - b * ey;
       cf = cmul2(aa, bb);
     }
-    img[2 * t] = make_double2(x, y);
-    img[2 * t + 1] = make_double2(wgt * cf.x, wgt * cf.y);
+    img[2 * t] = make_double2(x + 0.0 * (cf.x + cf.y), y);      // keeps a non-finite factor's NaN
+    reinterpret_cast<trig::PhaseOffset *>(img + 2 * t + 1)[0] = trig::phase_offset(cf.y, cf.x);
   }
   __syncwarp();
   bool finite = true;
@@ -539,23 +533,23 @@ c_kernel(const ObsDev *__restrict__ obs_arr, int oi, QCell cell, double2 *__rest
     const double yx = rs * tw[sidx].x, yy = -rs * tw[sidx].y;
     double2 v = make_double2(0.0, 0.0), d = v;
     for (int t = 0; t < npts; ++t) {
-      const double2 pt = img[2 * t], cf = img[2 * t + 1];
+      const double2 pt = img[2 * t];
+      const trig::PhaseOffset cf = *reinterpret_cast<const trig::PhaseOffset *>(img + 2 * t + 1);
       const double dx = pt.x - yx, dy = pt.y - yy;
       const double R2 = fma(dx, dx, fma(dy, dy, dz2));
-      const double iR = rsqrt(R2), kR = k * (R2 * iR);
-      double sn, cs;
-      c_sincos(kR, &sn, &cs);
+      const double iR = rsqrt(R2), R = R2 * iR, kR = k * R;
+      double sn, cs;                                   // of k R and the coefficient's phase
+      trig::sincos_phase(R, ph, cf, reinterpret_cast<const longlong2 *>(g_c_ring_q62), &sn, &cs);
       const double gr = cs * iR, gi = sn * iR;
       const double dc = axis == 0 ? dx : axis == 1 ? dy : dz;
       const double f = dc * (iR * iR);                 // (x - y)_c (ikR - 1) e^{ikR} / (4 pi P R^3)
-      const double hr = f * fma(-kR, gi, -gr), hi = f * fma(kR, gr, -gi);
-      v.x = fma(cf.x, gr, fma(-cf.y, gi, v.x));
-      v.y = fma(cf.x, gi, fma(cf.y, gr, v.y));
-      d.x = fma(cf.x, hr, fma(-cf.y, hi, d.x));
-      d.y = fma(cf.x, hi, fma(cf.y, hr, d.y));
+      v.x += gr;
+      v.y += gi;
+      d.x = fma(f, fma(-kR, gi, -gr), d.x);
+      d.y = fma(f, fma(kR, gr, -gi), d.y);
     }
-    sv[sidx] = v;
-    sd[sidx] = d;
+    sv[sidx] = make_double2(wgt * v.x, wgt * v.y);
+    sd[sidx] = make_double2(wgt * d.x, wgt * d.y);
   }
   __syncwarp();
   const long long r0 = (long long)(2 * grp) * nr + idx, r1 = r0 + nr;
