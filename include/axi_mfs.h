@@ -96,8 +96,9 @@ typedef enum {
  * computes c = V Sigma^+ U_R^H (Q^H fhat_n)_{1:N}, Sigma^+ keeping the
  * singular values >= 1e-10 sigma_max (the paper's truncation), as two
  * products and a scaling: the pseudo-inverse is never formed. The workspace
- * holds U_R, V and Sigma per mode (2 N^2 + N numbers). A mode whose Jacobi
- * sweeps do not converge in 40 latches AXI_ERR_TIMEOUT. */
+ * holds U_R, V and Sigma per mode (2 N^2 + N numbers) and N 32-bit integers.
+ * R is preconditioned by a QR with column pivoting (see axi_svd_jacobi). A
+ * mode whose Jacobi sweeps do not converge in 40 latches AXI_ERR_TIMEOUT. */
 #define AXI_PLAN_TSVD ((int32_t)1 << 17)
 
 typedef enum { AXI_SHAPE_POLAR = 0, AXI_SHAPE_CUP = 1 } axi_shape;
@@ -181,8 +182,9 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
  * integers:
  *   "next_update"   0 auto, 1 native FP64, 2 BF16 digits (split plans) for
  *                   the next panel's columns of each step;
- *   "panel_cluster" 0 auto (by the number of (obstacle, mode) tasks), or 1,
- *                   2, 4 CTAs per mode for the Householder panels;
+ *   "panel_cluster" 0 auto (by the panel's rows and the number of (obstacle,
+ *                   mode) tasks), or 1, 2, 4 CTAs per mode for the
+ *                   Householder panels;
  *   "rest_grid"     trailing updates of split plans: 0 auto (2 where the
  *                   update can read Y^H digits, i.e. the panel wrote its
  *                   reflector exponents, else 4), 1 mma.sync persistent (one
@@ -191,9 +193,9 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
  *                   same with one CTA per SM (room beside it for a panel or
  *                   next-panel CTA), 4 mma.sync with one CTA per (task,
  *                   column tile);
- *   "panel_threads" 0 auto (256 threads when a panel of more than 128 rows
- *                   runs on one CTA, else 128), 128 or 256 threads per
- *                   panel CTA;
+ *   "panel_threads" 0 auto (256 threads when a panel of 129 to 288 rows runs
+ *                   on one CTA and every task has an SM, else 128), 128 or
+ *                   256 threads per panel CTA;
  *   "crit_stream"   0 the panels and next-panel updates on `stream`, 1 on
  *                   a stream of the operator with the device's highest
  *                   priority (forked from and joined back into `stream`);
@@ -227,7 +229,8 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
  * the panel chain's choices together, then, for split plans, the next-panel
  * update's cluster, the fixed-point panel (128 and 256 threads) and the fill
  * chunk, each with the best so far ("rest_start" is left as given: 1 is
- * slower in a CUDA graph). It keeps the fastest in the plan, rebuilds the
+ * slower in a CUDA graph; the builds timed start their trailing updates as a
+ * captured graph does). It keeps the fastest in the plan, rebuilds the
  * operator with it and, when json_out is
  * not NULL, writes the choice with its build time ("build_ms"), the number
  * of candidates timed and the number skipped because they cannot run on this
@@ -406,14 +409,16 @@ axi_status axi_fill_c(const axi_operator *op, int32_t obs, const axi_cell *cell,
  * (m >= n >= 1, column-major, leading dimension lda >= m), in place: on
  * return d_A holds U Sigma (orthogonal columns), d_V (n x n, ldv >= n) the
  * right singular vectors and d_sigma[n] the singular values (column norms
- * of U Sigma, unsorted), so that A = (U Sigma) V^H. A sweep orders the
- * columns by decreasing norm (d_sigma holds that order during the call) and
- * rotates every column pair once (n' - 1 rounds of n'/2 disjoint pairs,
- * n' = n rounded up to even); the sweeps stop when every pair's |x^H y| / (||x|| ||y||) is at
- * most tol (e.g. 1e-15), after at most max_sweeps. *sweeps receives the
- * number run. The call synchronises `stream` after every sweep (not under
- * stream capture); calls that overlap on one device share the convergence
- * word. Device buffers are the caller's, 16-byte aligned (8 for d_sigma).
+ * of U Sigma, unsorted), so that A = (U Sigma) V^H. A is first factored by a
+ * Householder QR with column pivoting, A P = Q1 R1; the sweeps then rotate the
+ * columns of X = P R1^H, which are graded and nearly orthogonal, and end with
+ * X = V Sigma. A sweep orders the columns by decreasing norm (d_sigma holds
+ * that order during the call) and rotates every column pair once, by pairs of
+ * column blocks that meet in rounds of disjoint pairs; the sweeps stop when
+ * every pair's |x^H y| / (||x|| ||y||) is at most tol (e.g. 1e-15), after at
+ * most max_sweeps. *sweeps receives the number run. The call synchronises
+ * `stream` after the QR and after every sweep (not under stream capture).
+ * Device buffers are the caller's, 16-byte aligned (8 for d_sigma).
  * Errors: AXI_ERR_ARG, AXI_ERR_NUMERIC (not converged in max_sweeps, or a
  * non-finite value), AXI_ERR_CUDA.
  *
@@ -663,10 +668,15 @@ axi_status axi_eval_field(const axi_operator *op, int32_t obs, int32_t W,
  *   d_coef  : device [W][P][cols] coefficients (exterior field = first N columns).
  *   slices  : 0 = native FP64 direct sum; 4..7 = kernel values and strengths
  *             split into that many BF16 digits, contracted on tensor cores
- *             (the lattice's 90-degree symmetry is used when e_x = e_y and 4 | P).
+ *             (the lattice's 90-degree symmetry is used when e_x = e_y and 4 | P),
+ *             or, where a rule on the sizes expects it to be faster, the same sum
+ *             by spherical-wave expansions in FP64 about the obstacle's centre
+ *             (the images lie outside the sphere that holds the obstacle), to
+ *             about 2e-15 of the sum.
  *   d_out   : device [W][M*P], target index t = m*P + l.
  *   d_scratch, scratch_bytes : >= axi_near_image_workspace_bytes(); the split
- *             path stages kernel digits for blocks of whole target rings (~3 GB).
+ *             path stages kernel digits for blocks of whole target rings (~3 GB),
+ *             the expansions hold their coefficients (tens of MB).
  * Errors: AXI_ERR_ARG, AXI_ERR_UNSUPPORTED (slices), AXI_ERR_WORKSPACE, AXI_ERR_CUDA.
  */
 axi_status axi_near_image_workspace_bytes(const axi_operator *op, int32_t obs, int32_t W,

@@ -28,7 +28,7 @@ constexpr int kThreads = 256;
 // The shared-memory panel is bound by the FP64 pipe of one SM: 128 threads
 // (about two rows each) keep the per-warp reductions and scalar work small;
 // 256 threads give each SM sub-partition a second warp to cover the FP64
-// latency (the tuning chooses).
+// latency (launch_qr_panel has the rule).
 constexpr int kPanelThreads = 128;
 constexpr int kTN = 16;   // columns of the target per CTA in block-reflector kernels
 constexpr int kRC = 32;   // rows per shared-memory chunk
