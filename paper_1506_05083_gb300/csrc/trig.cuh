@@ -229,14 +229,17 @@ __device__ __forceinline__ void sincos_phase(double R, const RingPhase &p, Phase
   sincos_from_steps((long long)frac, step + (unsigned)(frac >> 63), tab, sp, cp);
 }
 
-// The phase of a unimodular factor, from its sine and cosine, as an offset.
+// The phase of a unimodular factor as an offset, from its sine and cosine: the
+// angle in (-pi, pi] in table steps as a nearest integer and a signed remainder,
+// so that a negative angle below the last bit of a step stays next to zero (a
+// floor and its remainder would round to a whole step there).
 __device__ __forceinline__ PhaseOffset phase_offset(double sn, double cs) {
-  // from its sine and cosine: the angle in (-pi, pi] in table steps
   const double steps = atan2(sn, cs) * 162.97466172610083;
-  const double fl = floor(steps);
+  const double n = rint(steps);
+  const long long r = (long long)((steps - n) * 0x1p63);   // |steps - n| <= 1/2: within +-2^62
   PhaseOffset o;
-  o.step = (unsigned)(int)fl;
-  o.frac = (unsigned long long)((steps - fl) * 0x1p53) << 11;
+  o.step = (unsigned)((int)n - (r < 0 ? 1 : 0));
+  o.frac = (unsigned long long)r << 1;
   return o;
 }
 
