@@ -755,31 +755,54 @@ size_t sph_layout(const ObsDev &h, int W, int p, int ncls, char *base, SphBuf *b
 
 int sph_classes(double ex, double ey) { return ex == ey ? 2 : 3; }
 
+// One function a kernel, so that a kernel has one record of the shared memory it
+// was granted: a second record (one per wave tile below) would let a smaller
+// grant replace a larger one that the first still counts on.
+cudaError_t launch_setup(const ObsDev *d_o, const SphArgs &g, const SphBuf &b, const double *dirs,
+                         cudaStream_t st) {
+  const int p = g.p, L = 2 * p + 1, parts = (p / 2 + 1 + kTabWarps - 1) / kTabWarps;
+  const int blocks = g.ncls + 4 + ((g.M + 31) / 32 + (g.N + 31) / 32) * parts + p + 1;
+  const size_t table = sizeof(double) * ((size_t)(p + 2) * 32 + (size_t)kTabWarps * 6 * (p + 1));
+  const size_t smem = std::max(table, sizeof(double) * ((size_t)3 * L + 1));
+  static size_t granted = 0;
+  const cudaError_t e = ensure_dynamic_smem(sph_setup_kernel, smem, granted);
+  if (e != cudaSuccess) return e;
+  sph_setup_kernel<<<blocks, kSetupThreads, smem, st>>>(d_o, g, b, dirs, parts);
+  return cudaGetLastError();
+}
+
+template <int TP>
+cudaError_t launch_p2m(const SphArgs &g, const SphBuf &b, const double2 *coef, cudaStream_t st) {
+  const int p = g.p, L = 2 * p + 1;
+  const size_t block = sizeof(double) * (3 * L + 1) + 3 * sizeof(double2) * L;
+  const size_t tile = sizeof(double) * 32 * 33 + sizeof(double2) * 32 * 2 * TP;
+  const size_t smem = std::max(block, tile);
+  static size_t granted = 0;
+  const cudaError_t e = ensure_dynamic_smem(sph_p2m_kernel<TP>, smem, granted);
+  if (e != cudaSuccess) return e;
+  sph_p2m_kernel<TP><<<dim3(p + 1, g.ncls + (p + 32) / 32 * ((g.W + TP - 1) / TP)), kMatThreads, smem, st>>>(
+      g, b, coef);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dft(const ObsDev *d_o, const SphArgs &g, const SphBuf &b, double2 *U, cudaStream_t st) {
+  const size_t smem = sizeof(double2) * ((size_t)g.P + (g.P + 1) / 2 + (size_t)kDftSeq * g.P);
+  static size_t granted = 0;
+  const cudaError_t e = ensure_dynamic_smem(sph_dft_kernel, smem, granted);
+  if (e != cudaSuccess) return e;
+  sph_dft_kernel<<<dim3((g.M + kDftSeq - 1) / kDftSeq, g.W), 32 * kDftSeq, smem, st>>>(d_o, g, b.modes, U);
+  return cudaGetLastError();
+}
+
 template <int TC>
-cudaError_t sph_launch(const ObsDev *d_o, const ObsDev &h, const SphArgs &g, const SphBuf &b,
+cudaError_t sph_launch(const ObsDev *d_o, const SphArgs &g, const SphBuf &b,
                        const double2 *coef, const double *dirs, double2 *U, cudaStream_t st) {
-  const int p = g.p, L = 2 * p + 1, wt = (g.W + TC - 1) / TC;
+  const int p = g.p, wt = (g.W + TC - 1) / TC;
   const int slabs = (p + kMatThreads / TC) / (kMatThreads / TC);   // of the rows 0 .. p
   cudaError_t e;
-  {
-    const int parts = (p / 2 + 1 + kTabWarps - 1) / kTabWarps;
-    const int blocks = g.ncls + 4 + ((g.M + 31) / 32 + (g.N + 31) / 32) * parts + p + 1;
-    const size_t table = sizeof(double) * ((size_t)(p + 2) * 32 + (size_t)kTabWarps * 6 * (p + 1));
-    const size_t smem = std::max(table, sizeof(double) * ((size_t)3 * L + 1));
-    static size_t granted = 0;
-    if ((e = ensure_dynamic_smem(sph_setup_kernel, smem, granted)) != cudaSuccess) return e;
-    sph_setup_kernel<<<blocks, kSetupThreads, smem, st>>>(d_o, g, b, dirs, parts);
-  }
-  {
-    const size_t block = sizeof(double) * (3 * L + 1) + 3 * sizeof(double2) * L;
-    constexpr int TP = TC < 4 ? TC : 4;    // finer tiles: the orders' degree ranges are uneven
-    const size_t tile = sizeof(double) * 32 * 33 + sizeof(double2) * 32 * 2 * TP;
-    const size_t smem = std::max(block, tile);
-    static size_t granted = 0;
-    if ((e = ensure_dynamic_smem(sph_p2m_kernel<TP>, smem, granted)) != cudaSuccess) return e;
-    sph_p2m_kernel<TP><<<dim3(p + 1, g.ncls + (p + 32) / 32 * ((g.W + TP - 1) / TP)), kMatThreads, smem, st>>>(
-        g, b, coef);
-  }
+  constexpr int TP = TC < 4 ? TC : 4;      // finer tiles: the orders' degree ranges are uneven
+  if ((e = launch_setup(d_o, g, b, dirs, st)) != cudaSuccess) return e;
+  if ((e = launch_p2m<TP>(g, b, coef, st)) != cudaSuccess) return e;
   {
     const size_t smem = 2 * sizeof(double2) * (p + 1) * TC;
     static size_t granted = 0;
@@ -804,11 +827,7 @@ cudaError_t sph_launch(const ObsDev *d_o, const ObsDev &h, const SphArgs &g, con
     if ((e = ensure_dynamic_smem(sph_l2p_kernel<TC>, smem, granted)) != cudaSuccess) return e;
     sph_l2p_kernel<TC><<<dim3(g.P, (g.M + 31) / 32, wt), kMatThreads, smem, st>>>(g, b);
   }
-  const size_t smem = sizeof(double2) * ((size_t)g.P + (g.P + 1) / 2 + (size_t)kDftSeq * g.P);
-  static size_t granted = 0;
-  if ((e = ensure_dynamic_smem(sph_dft_kernel, smem, granted)) != cudaSuccess) return e;
-  sph_dft_kernel<<<dim3((g.M + kDftSeq - 1) / kDftSeq, g.W), 32 * kDftSeq, smem, st>>>(d_o, g, b.modes, U);
-  return cudaGetLastError();
+  return launch_dft(d_o, g, b, U, st);
 }
 
 }  // namespace
@@ -878,10 +897,10 @@ cudaError_t launch_near_sph(const ObsDev *d_o, const ObsDev &h, int W, const dou
   SphBuf b;
   sph_layout(h, W, p, g.ncls, static_cast<char *>(scratch), &b);
   switch (wave_tile(W)) {
-    case 1: return sph_launch<1>(d_o, h, g, b, coef, dirs, U, st);
-    case 2: return sph_launch<2>(d_o, h, g, b, coef, dirs, U, st);
-    case 4: return sph_launch<4>(d_o, h, g, b, coef, dirs, U, st);
-    default: return sph_launch<8>(d_o, h, g, b, coef, dirs, U, st);
+    case 1: return sph_launch<1>(d_o, g, b, coef, dirs, U, st);
+    case 2: return sph_launch<2>(d_o, g, b, coef, dirs, U, st);
+    case 4: return sph_launch<4>(d_o, g, b, coef, dirs, U, st);
+    default: return sph_launch<8>(d_o, g, b, coef, dirs, U, st);
   }
 }
 
