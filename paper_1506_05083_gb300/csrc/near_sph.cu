@@ -240,8 +240,10 @@ __device__ void delta_matrix(int l, double *__restrict__ out, double *sh) {
   }
 }
 
-// h_l(x), l = 0 .. 2p, of one distance: y_l upwards and j_l by Miller's
-// recurrence, one thread each.
+// h_l(x), l = 0 .. 2p, of one distance, one thread each: y_l upwards; j_l upwards
+// too where x is beyond the last degree (stable for l < x), else by Miller's
+// recurrence from 40 degrees past the last one and the turning zone (a few
+// x^{1/3} wide). At most 370 steps either way, whatever the period.
 __device__ void hankel_row(double x, int p, double2 *__restrict__ out, double *sh) {
   const int L = 2 * p + 1;
   double *c = sh, *yl = c + L + 1, *jl = yl + L;            // c: (2l + 1) / x
@@ -258,8 +260,16 @@ __device__ void hankel_row(double x, int p, double2 *__restrict__ out, double *s
       y0 = y1;
       y1 = y2;
     }
+  } else if (threadIdx.x == 32 && x > L) {
+    double j0 = sn * ix, j1 = (j0 - cs) * ix;
+    for (int l = 0; l < L; ++l) {
+      jl[l] = j0;
+      const double j2 = fma(c[l + 1], j1, -j0);
+      j0 = j1;
+      j1 = j2;
+    }
   } else if (threadIdx.x == 32) {
-    const int L0 = L + (int)x + 40;
+    const int L0 = max(L, (int)(x + 12.0 * cbrt(x))) + 40;
     double f1 = 0.0, f0 = 1.0;
     for (int l = L0; l >= 1; --l) {
       const double fm = fma(l <= L ? c[l] : (2.0 * l + 1.0) * ix, f0, -f1);
@@ -837,11 +847,15 @@ cudaError_t sph_launch(const ObsDev *d_o, const SphArgs &g, const SphBuf &b,
 // (2l + 1) j_l(k r_s) h_l(k (D - r_t)) and (2l + 1) j_l(k r_t) h_l(k (D - r_s)),
 // with the derivative's factor l, below 2^-58 of the largest. D is the shorter
 // period. Refused: p above kSphMaxDegree (an image too close, or very large
-// k r), coefficients h_2p(kD) beyond the FP64 range (k D far below 1), and
-// targets on the axis, where the derivative's recurrence divides by sin(theta).
+// k r), coefficients h_2p(kD) beyond the FP64 range (k D far below 1), k D of 2^19
+// and more (the recurrences were compared with quadruple precision up to 7e5),
+// and targets on the axis, where the derivative's recurrence divides by
+// sin(theta).
 int near_sph_degree(const ObsDev &h, double ex, double ey) {
   const double D = std::min(ex, ey), rs = h.sph_rs, rt = h.sph_rt;
   if (!(rs > 0.0) || !(rt > 0.0) || !(h.sph_rho_min > 1e-6 * rt) || !(D > 1.02 * (rs + rt))) return 0;
+  const double r = std::max(rs, rt);
+  if (!(h.k * r < kSphMaxDegree) || !(h.k * std::hypot(ex, ey) < 0x1p19) || !(h.k * (D - r) > 0x1p-100)) return 0;
   constexpr int L = 2 * kSphMaxDegree + 2;
   int ja[L + 1], jb[L + 1], ha[L + 1], hb[L + 1];
   constexpr int L1 = kSphMaxDegree + 1;

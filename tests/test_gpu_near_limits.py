@@ -1,9 +1,10 @@
 """The near-image expansions at the limits of their rules: shared-memory grants of
-calls of several sizes in one process."""
+calls of several sizes in one process, and lattices whose images are far away."""
 import numpy as np
 import pytest
 
 import synth
+from test_gpu_near_sph import _abs_sum
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -31,3 +32,28 @@ def test_near_sizes_one_after_another():
         small = near(W, 3.1)
         assert torch.equal(near(9, 2.78), large), W
         assert torch.equal(near(W, 3.1), small), W
+
+
+def _against_direct(op, k, lat, c, slices):
+    """Error of a split call against the direct FP64 sum, relative to sum |K| |sigma|."""
+    from paper_1506_05083_gb300 import axi
+    spec = op.specs[0]
+    d = torch.tensor(synth.plane_wave_directions(c.shape[0], 3), device="cuda")
+    ct = torch.tensor(c, device="cuda")
+    ref = axi.near_image_sum(op, ct, lat, d, slices=0)
+    U = axi.near_image_sum(op, ct, lat, d, slices=slices)
+    return (U - ref).abs().max().item() / _abs_sum(k, spec.coll, spec.src, c[:, :, :spec.N], lat, spec.P)
+
+
+@pytest.mark.parametrize("lat", [(30.0, 30.0), (3.0e3, 3.0e3), (2.0e5, 9.0e4), (4.0, 1.0e5), (2.0e6, 2.0e6)])
+def test_near_far_lattices(lat):
+    """Periods from ten to a million body sizes, where h_l(k D) runs upwards (k D beyond
+    every degree) and beyond k D = 2^19, where the direct split sum serves. Tolerance: that
+    of the other lattices, 1.5e-13, and the phases: k, D and R enter both sums with four
+    roundings of k D radians."""
+    k, N, P = 3.0, 30, 18
+    op = _operator(N, P, k)
+    rng = np.random.default_rng(5)
+    c = rng.standard_normal((2, P, N)) + 1j * rng.standard_normal((2, P, N))
+    err = _against_direct(op, k, lat, c, 7)
+    assert err < 1.5e-13 + 4 * 2.0 ** -53 * k * np.hypot(*lat), err
