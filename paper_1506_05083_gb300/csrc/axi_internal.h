@@ -350,8 +350,9 @@ cudaError_t launch_near_image(const ObsDev *d_o, const ObsDev &h, int W, const d
                               double ex, double ey, const double *dirs, int slices, double2 *U,
                               void *scratch, cudaStream_t st);
 // near_sph.cu: the near-image sum by spherical-wave expansions. Degree of the
-// expansions for a lattice (0: not usable, the direct sum runs), scratch, launch.
-int near_sph_degree(const ObsDev &h, double ex, double ey);
+// expansions for a lattice and the digits asked for (0: not usable, the direct
+// sum runs), scratch, launch.
+int near_sph_degree(const ObsDev &h, double ex, double ey, int slices);
 double near_sph_estimate_us(const ObsDev &h, int W, int p);
 size_t near_sph_scratch_bytes(const ObsDev &h, int W, double ex, double ey, int p);
 cudaError_t launch_near_sph(const ObsDev *d_o, const ObsDev &h, int W, const double2 *coef, double ex,

@@ -452,7 +452,7 @@ int block_targets(const ObsDev &h, int W, int nrot) {
 // The direct FP64 sum (slices 0) stays what it says.
 int near_degree(const ObsDev &h, const NearGeom &g, int slices) {
   if (slices <= 0) return 0;
-  const int p = near_sph_degree(h, g.ex, g.ey);
+  const int p = near_sph_degree(h, g.ex, g.ey, slices);
   if (p == 0) return 0;
   const double direct = g.nrep * (80.0 + 1.45e-4 * g.S * ((double)h.M * h.P));
   return near_sph_estimate_us(h, g.W, p) < direct ? p : 0;

@@ -44,9 +44,15 @@
 // J. Sci. Comput. 25 (2003)), started from Gegenbauer's addition theorem for
 // h_m(kR)/(kR)^m (the distance from the axis is the same in both frames):
 //   T^m_{l,m} = sqrt((2m+1)!!/(2m)!! (2l+1) (l+m)!/(l-m)!) h_l(kD) / (kD)^m.
-// Run upwards in n the recurrence follows its dominant solution: against
-// 60-digit arithmetic the error is 3e-16 of the largest entry (weighted by the
-// waves' sizes) for kD = 8 .. 82, p up to 85. T depends on |m|, and
+// Run upwards in n the recurrence loses digits at large k r where p nears kD
+// (orders m of 4 to 16): against quadruple precision the error of one source's
+// field, relative to the largest kernel value, over periods of 1.3 to 60 times
+// r_s + r_t is below 2e-14 for k r = 20, 3e-14 for 35, 5e-14 for 45, 3e-13 for 55 and
+// 1e-12 for 60 (k r is that of the larger radius). Measured, single sources at 1.3
+// (r_s + r_t), against the direct sum of 7 digits: 6e-15 and 7e-15 for k r = 20, 1.7e-14
+// and 1.0e-14 for 33, 2.0e-14 and 1.6e-14 for 45, 1.6e-13 and 1.7e-14 for 57; 6 digits
+// keep 5e-13. So a caller who asks for 7 digits takes this path up to k r = 35,
+// with fewer up to 55 (near_sph_degree). T depends on |m|, and
 // M'_{-m}(-c) = (-1)^l M'_m(c), so the sums over even and odd l' give (m, c)
 // and (-m, -c) together.
 #include <algorithm>
@@ -847,15 +853,16 @@ cudaError_t sph_launch(const ObsDev *d_o, const SphArgs &g, const SphBuf &b,
 // (2l + 1) j_l(k r_s) h_l(k (D - r_t)) and (2l + 1) j_l(k r_t) h_l(k (D - r_s)),
 // with the derivative's factor l, below 2^-58 of the largest. D is the shorter
 // period. Refused: p above kSphMaxDegree (an image too close, or very large
-// k r), coefficients h_2p(kD) beyond the FP64 range (k D far below 1), k D of 2^19
+// k r), k r beyond what the translation keeps of the caller's digits (the note at
+// the head of this file), coefficients h_2p(kD) beyond the FP64 range (k D far below 1), k D of 2^19
 // and more (the recurrences were compared with quadruple precision up to 7e5),
 // and targets on the axis, where the derivative's recurrence divides by
 // sin(theta).
-int near_sph_degree(const ObsDev &h, double ex, double ey) {
+int near_sph_degree(const ObsDev &h, double ex, double ey, int slices) {
   const double D = std::min(ex, ey), rs = h.sph_rs, rt = h.sph_rt;
   if (!(rs > 0.0) || !(rt > 0.0) || !(h.sph_rho_min > 1e-6 * rt) || !(D > 1.02 * (rs + rt))) return 0;
   const double r = std::max(rs, rt);
-  if (!(h.k * r < kSphMaxDegree) || !(h.k * std::hypot(ex, ey) < 0x1p19) || !(h.k * (D - r) > 0x1p-100)) return 0;
+  if (!(h.k * r <= (slices >= 7 ? 35.0 : 55.0)) || !(h.k * std::hypot(ex, ey) < 0x1p19) || !(h.k * (D - r) > 0x1p-100)) return 0;
   constexpr int L = 2 * kSphMaxDegree + 2;
   int ja[L + 1], jb[L + 1], ha[L + 1], hb[L + 1];
   constexpr int L1 = kSphMaxDegree + 1;

@@ -1,5 +1,6 @@
 """The near-image expansions at the limits of their rules: shared-memory grants of
-calls of several sizes in one process, and lattices whose images are far away."""
+calls of several sizes in one process, lattices whose images are far away, and
+large k r."""
 import numpy as np
 import pytest
 
@@ -57,3 +58,28 @@ def test_near_far_lattices(lat):
     c = rng.standard_normal((2, P, N)) + 1j * rng.standard_normal((2, P, N))
     err = _against_direct(op, k, lat, c, 7)
     assert err < 1.5e-13 + 4 * 2.0 ** -53 * k * np.hypot(*lat), err
+
+
+@pytest.mark.parametrize("kr,slices", [(34.0, 7), (57.0, 7), (54.0, 6), (60.0, 6), (34.0, 4)])
+def test_near_large_kr(kr, slices):
+    """One source a wave, so that the error is relative to single kernel values: a
+    split call keeps the digits it was asked for, 2^(-7 slices + 5), whether the
+    expansions (whose translation loses digits as k r grows) or the direct sum serves.
+    Three waves a call, where the expansions are expected to be the faster."""
+    from paper_1506_05083_gb300 import axi
+    N, P = 30, 18
+    spec = _operator(N, P, 1.0).specs[0]
+    z = np.linspace(-0.3, 0.3, 6001)                        # centre of the smallest sphere
+    rad = lambda a: np.hypot(a[:, 0], a[:, 1] - z[:, None]).max(1)  # noqa: E731
+    zc = np.argmin(np.maximum(rad(spec.coll), rad(spec.src)))
+    rs, rt = rad(spec.src)[zc], rad(spec.coll)[zc]
+    k, D = kr / rt, 1.3 * (rs + rt)
+    op = axi.Operator([axi.ObstacleSpec(spec.bc, spec.M, N, P, spec.q, k, 0.0, spec.coll, spec.src)])
+    worst = 0.0
+    for j in range(0, N, 3):
+        c = np.zeros((3, P, N), dtype=complex)
+        for w in range(3):
+            c[w, :, j + w] = 1.0                            # all modes alike: the ring's node at angle 0
+        worst = max(worst, _against_direct(op, k, (D, D), c, slices))
+    print(f"k r {kr}, {slices} digits: {worst:.2e}")
+    assert worst < 2.0 ** (-7 * slices + 5)
