@@ -57,6 +57,7 @@
 // and (-m, -c) together.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "axi_internal.h"
 #include "fft.cuh"
@@ -116,6 +117,10 @@ constexpr int kSetupThreads = 32 * kTabWarps;
 // j_l(kr) Pbar_l^m or its normal derivative, out[(sph_off(m) + l - m) n + i].
 // Miller's backward recurrence for j_l (as btilde_kernel), three-term
 // recurrences for Pbar; the FP64 pipe bounds it (about 8 operations an entry).
+// dPbar_l^m/dtheta is (l cos Pbar_l - c Pbar_{l-1}) / sin for m > 0, where both
+// terms fall with sin^m; for m = 0 it would subtract nearly equal terms near the
+// axis, so there -sin Pbar_l' with P_l' = P_{l-2}' + (2l - 1) P_{l-1}, a sum of
+// like signs near the axis.
 template <bool DERIV>
 __device__ void wave_table(const double *__restrict__ pts, int stride, int n, double k, double zc, int p,
                            int grp, int part, double *__restrict__ out, double *sh) {
@@ -170,7 +175,9 @@ __device__ void wave_table(const double *__restrict__ pts, int stride, int n, do
         a = sqrt((4.0 * ll - 1.0) / (ll - mm));
         b = sqrt((l1 - mm) / (4.0 * l1 - 1.0));
       }
-      if (DERIV && l > m) cc = sqrt((2.0 * l + 1.0) * (l - m) * (l + m) / (2.0 * l - 1.0));
+      if (DERIV && l > m)
+        cc = m > 0 ? sqrt((2.0 * l + 1.0) * (l - m) * (l + m) / (2.0 * l - 1.0))
+                   : l > 2 ? sqrt((2.0 * l + 1.0) / (2.0 * l - 3.0)) : 0.0;      // of Pbar_{l-2}'
       c[l] = a;
       c[(p + 1) + l] = b;
       c[2 * (p + 1) + l] = cc;
@@ -196,24 +203,40 @@ __device__ void wave_table(const double *__restrict__ pts, int stride, int n, do
     }
     double cur = ((m & 1) ? -sqrt(prod) : sqrt(prod)) * spow, prev = 0.0, dl = m;   // dl = l
     double *blk = out + (size_t)sph_off(m, p) * n;
-    for (int l = m; l <= p; ++l) {
-      if (l > m) {
-        const double nxt = ca[l] * fma(ct, cur, -cb[l] * prev);
-        prev = cur;
-        cur = nxt;
-        dl += 1.0;
+    auto column = [&](auto zonal) {                         // two loops: no instruction of the other form
+      double q0 = 0.0, q1 = 0.0;                            // m = 0: Pbar_l', Pbar_{l-1}'
+      for (int l = m; l <= p; ++l) {
+        if (l > m) {
+          const double nxt = ca[l] * fma(ct, cur, -cb[l] * prev);
+          prev = cur;
+          cur = nxt;
+          dl += 1.0;
+          if constexpr (DERIV && zonal.value) {
+            const double q2 = fma(dl * ca[l], prev, cc[l] * q1);
+            q1 = q0;
+            q0 = q2;
+          }
+        }
+        const double j = jl[l * 32 + lane];
+        double v;
+        if constexpr (DERIV) {
+          double dP;
+          if constexpr (zonal.value)
+            dP = -st * q0;
+          else
+            dP = fma(dl * ct, cur, -cc[l] * prev) * ist;
+          const double dj = l == 0 ? -jl[32 + lane] : fma(-(dl + 1.0) * ix, j, jl[(l - 1) * 32 + lane]);
+          v = fma(Ak * dj, cur, Bk * j * dP);
+        } else {
+          v = j * cur;
+        }
+        if (live) blk[(size_t)(l - m) * n + i] = v;
       }
-      const double j = jl[l * 32 + lane];
-      double v;
-      if (DERIV) {
-        const double dP = fma(dl * ct, cur, -cc[l] * prev) * ist;
-        const double dj = l == 0 ? -jl[32 + lane] : fma(-(dl + 1.0) * ix, j, jl[(l - 1) * 32 + lane]);
-        v = fma(Ak * dj, cur, Bk * j * dP);
-      } else {
-        v = j * cur;
-      }
-      if (live) blk[(size_t)(l - m) * n + i] = v;
-    }
+    };
+    if (DERIV && m == 0)
+      column(std::true_type{});
+    else
+      column(std::false_type{});
   }
 }
 

@@ -83,3 +83,22 @@ def test_near_large_kr(kr, slices):
         worst = max(worst, _against_direct(op, k, (D, D), c, slices))
     print(f"k r {kr}, {slices} digits: {worst:.2e}")
     assert worst < 2.0 ** (-7 * slices + 5)
+
+
+@pytest.mark.parametrize("rho", [2e-6, 1e-5, 1e-3, 0.05])
+def test_near_ring_close_to_the_axis(rho):
+    """Rings next to the axis with oblique normals (the tip of a cone), where the normal
+    derivative has a theta part of its own size: the tolerance of the other lattices,
+    1.5e-13 of sum |K| |sigma|."""
+    from paper_1506_05083_gb300 import axi
+    N, P, k = 30, 18, 4.0
+    spec = _operator(N, P, k).specs[0]
+    coll = spec.coll.copy()
+    coll[0, 0] = coll[-1, 0] = rho
+    coll[0, 2:] = [0.8, 0.6]
+    coll[-1, 2:] = [0.6, -0.8]
+    op = axi.Operator([axi.ObstacleSpec(spec.bc, spec.M, N, P, spec.q, k, 0.0, coll, spec.src)])
+    rng = np.random.default_rng(9)
+    c = rng.standard_normal((3, P, N)) + 1j * rng.standard_normal((3, P, N))
+    err = _against_direct(op, k, (3.4, 3.4), c, 7)
+    assert err < 1.5e-13, err
