@@ -6,8 +6,10 @@
 //   c = V Sigma^+ U_R^H (Q^H fhat_n)_{1:N},
 // Sigma^+ keeping the singular values >= 1e-10 sigma_max.
 //
-// R's SVD is the batched block Jacobi of svd_dense.cu. Blocks too wide for its
-// shared memory (n above 3400) take the kernel below, one CTA per mode.
+// R's SVD is the batched block Jacobi of svd_dense.cu, a chain of some 230 launches
+// at the least. Blocks up to 23 columns (kSmallBlock) take the kernel below, one CTA
+// per mode and one launch, and so do blocks too wide for the other's shared memory
+// (n above 3400).
 //
 // One-sided (Hestenes) Jacobi: the columns g_i of G (initially R) are made
 // mutually orthogonal by plane rotations from the right, G <- G J, V <- V J.
@@ -28,6 +30,11 @@ namespace {
 
 constexpr int kJThreads = 512;
 constexpr int kMaxSweeps = 40;
+// Widest block of the one-CTA kernel. Builds by it and by the batch (ms; 5, 13, 41
+// and 81 modes differ little by it): 8 columns 0.32 and 1.11, 16 columns 1.10 and
+// 1.75, 20 columns 1.87 and 2.02, 23 columns 2.41 and 2.22 to 2.52, 24 columns 2.60 and 2.30
+// to 2.60, 32 columns 5.37 and 3.45.
+constexpr int kSmallBlock = 23;
 constexpr double kEps = 2.220446049250313e-16;
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -260,7 +267,7 @@ tsvd_apply_kernel(const ObsDev *__restrict__ od, double2 *__restrict__ X, int nc
 }  // namespace
 
 cudaError_t launch_tsvd(const ObsDev *d_o, const ObsDev &h, cudaStream_t st) {
-  if (svd_batch_fits(h.cols, h.cols)) {
+  if (h.cols > kSmallBlock && svd_batch_fits(h.cols, h.cols)) {
     const long long n = h.cols;
     tsvd_copy_r_kernel<<<dim3((unsigned)((n * n + 255) / 256), h.D), 256, 0, st>>>(d_o);
     const SvdBatch q{h.svdU, n, n * n, h.svdV, n, n * n, h.svdS, n, h.svdSweeps, h.mode_owned, h.cols, h.cols};

@@ -96,3 +96,11 @@ def test_svd_long_columns(m, n, kind):
         assert np.abs(np.sort(sg) / ref - 1).max() < 1e-13
     assert np.abs(Vn.conj().T @ Vn - np.eye(n)).max() < 1e-13
     assert np.abs(US @ Vn.conj().T - A).max() < 1e-13 * ref[-1]
+
+
+@pytest.mark.parametrize("N,P", [(1, 4), (2, 8), (13, 8), (23, 40), (24, 40)])
+def test_tsvd_small_blocks(N, P):
+    """Truncated-SVD blocks on either side of the width from which they are a batch:
+    test_tsvd_blocks's checks and tolerances."""
+    import test_gpu_svd_blocks as blocks
+    blocks.test_tsvd_blocks(N, P)
