@@ -216,7 +216,9 @@ axi_status axi_plan_create(const axi_obstacle *obs, int32_t n_obs, int32_t prec,
  *                   starts as soon as the panel (and its digits) is done,
  *                   beside the next-panel update; launched directly it starts
  *                   after the next-panel update, so that it runs beside the
- *                   next panel only; 1 always after the next-panel update;
+ *                   next panel only, except in split plans with at most a
+ *                   fifth as many modes as the device has SMs; 1 always after
+ *                   the next-panel update;
  *   "apply_cluster" split plans' Q^H in axi_apply_operator: 0 auto (4 CTAs
  *                   per (mode, 32-column tile) when all of them fit in one
  *                   wave of two CTAs per SM, else 2), or 2, 4.

@@ -747,14 +747,18 @@ static axi_status run_build(axi_operator_s *op, cudaStream_t st,
       return AXI_ERR_CUDA;
     st = op->crit;
   }
-  // Start of the trailing updates (Tuning::rest_start). Launched directly with
-  // the queue full, an update that is ready together with the next-panel update
-  // fills the SMs first and the panel chain waits; a captured graph orders the
-  // two well and gains from the overlap. Builds launched back to back, early
-  // against late: cup 15.5 and 13.9 ms, smooth body 3.5 and 3.0, transmission body
-  // 6.9 and 6.5; as a graph: 13.2 and 14.4, 2.75 and 3.26, 7.3 and 7.8.
+  // Start of the trailing updates (Tuning::rest_start). Launched directly, an update
+  // that is ready together with the next-panel update can fill the SMs first while
+  // the panel chain waits; a captured graph orders the two well and gains from the
+  // overlap (cup, early against late: 13.2 and 14.4 ms, smooth body 2.75 and 3.26).
+  // A split plan with few modes leaves SMs to both either way and starts early as
+  // well. Solves with several operators in the process, early against late (ms): 17
+  // modes of 320 proxies 6.19 and 6.42, 25 modes of 160 2.49 and 2.57, 33 modes of 160
+  // 2.67 and 2.60, 41 modes of 240 5.29 and 4.85; native plans gain at every number
+  // (builds of 9 modes of 240 proxies 4.51 and 3.38, of 121 modes 14.5 and 13.9).
   bool late = p->tune.rest_start == 1;
-  if (!late && !as_graph) {
+  const bool few = slices > 0 && !p->step_tasks.empty() && 5 * p->step_tasks[0] <= axi::sm_count();
+  if (!late && !as_graph && !few) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) late = cap == cudaStreamCaptureStatusNone;
     else (void)cudaGetLastError();

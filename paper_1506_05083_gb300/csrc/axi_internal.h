@@ -35,8 +35,9 @@ struct Tuning {
   int panel_fixed = 0;    // split plans' panel: 0 auto (FP64), 1 FP64, 2 fixed point (one CTA per
                           // mode)
   int rest_start = 0;     // trailing update of a step: 0 automatic (after the panel's digits, beside
-                          // the next-panel update, in a captured graph; after the next-panel update
-                          // when launched directly), 1 always after the next-panel update
+                          // the next-panel update, in a captured graph and in split plans with few
+                          // modes; else after the next-panel update when launched directly), 1
+                          // always after the next-panel update
   int apply_cluster = 0;  // split Q^H of the apply: CTAs per (mode, column tile) cluster,
                           // 0 auto (4 when every cluster fits in one wave of CTAs, else 2)
 };
