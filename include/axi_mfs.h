@@ -676,9 +676,11 @@ axi_status axi_eval_field(const axi_operator *op, int32_t obs, int32_t W,
  *             (the images lie outside the sphere that holds the obstacle), to
  *             about 2e-15 of the sum.
  *   d_out   : device [W][M*P], target index t = m*P + l.
- *   d_scratch, scratch_bytes : >= axi_near_image_workspace_bytes(); the split
- *             path stages kernel digits for blocks of whole target rings (~3 GB),
- *             the expansions hold their coefficients (tens of MB).
+ *   d_scratch, scratch_bytes : >= axi_near_image_workspace_bytes() for this
+ *             lattice and slices and for W or more waves; the split path stages
+ *             kernel digits for blocks of whole target rings (~3 GB), the
+ *             expansions hold their coefficients (tens of MB), and a scratch that
+ *             holds only one of the two takes that one.
  * Errors: AXI_ERR_ARG, AXI_ERR_UNSUPPORTED (slices), AXI_ERR_WORKSPACE, AXI_ERR_CUDA.
  */
 axi_status axi_near_image_workspace_bytes(const axi_operator *op, int32_t obs, int32_t W,

@@ -1198,11 +1198,11 @@ axi_status axi_near_image_sum(const axi_operator *op, int32_t obs, int32_t W, co
   if (slices != 0 && (slices < 4 || slices > 7)) return AXI_ERR_UNSUPPORTED;
   if (!(lattice->ex > 0) || !(lattice->ey > 0)) return AXI_ERR_ARG;
   const ObsDev &d = op->plan->obs[obs].dev;
-  if (scratch_bytes < axi::near_image_scratch_bytes(d, W, lattice->ex, lattice->ey, slices))
-    return AXI_ERR_WORKSPACE;
+  const int way = axi::near_image_way(d, W, lattice->ex, lattice->ey, slices, scratch_bytes);
+  if (way < 0) return AXI_ERR_WORKSPACE;
   return cuda_status(axi::launch_near_image(op->d_obs + obs, d, W,
                                             reinterpret_cast<const double2 *>(d_coef),
-                                            lattice->ex, lattice->ey, d_dirs, slices,
+                                            lattice->ex, lattice->ey, d_dirs, slices, way,
                                             reinterpret_cast<double2 *>(d_out), d_scratch,
                                             static_cast<cudaStream_t>(stream)));
 }

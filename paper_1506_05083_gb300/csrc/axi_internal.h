@@ -347,8 +347,9 @@ cudaError_t launch_rhs_fft(const ObsDev *d_o, const ObsDev &h_o, int W, const do
 cudaError_t launch_point_fft(const ObsDev *d_o, const ObsDev &h_o, int W, const double2 *coef,
                              double2 *sigma, cudaStream_t st);
 size_t near_image_scratch_bytes(const ObsDev &h, int W, double ex, double ey, int slices);
+int near_image_way(const ObsDev &h, int W, double ex, double ey, int slices, size_t bytes);
 cudaError_t launch_near_image(const ObsDev *d_o, const ObsDev &h, int W, const double2 *coef,
-                              double ex, double ey, const double *dirs, int slices, double2 *U,
+                              double ex, double ey, const double *dirs, int slices, int way, double2 *U,
                               void *scratch, cudaStream_t st);
 // near_sph.cu: the near-image sum by spherical-wave expansions. Degree of the
 // expansions for a lattice and the digits asked for (0: not usable, the direct

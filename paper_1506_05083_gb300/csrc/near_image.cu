@@ -458,13 +458,9 @@ int near_degree(const ObsDev &h, const NearGeom &g, int slices) {
   return near_sph_estimate_us(h, g.W, p) < direct ? p : 0;
 }
 
-}  // namespace
-
-size_t near_image_scratch_bytes(const ObsDev &h, int W, double ex, double ey, int slices) {
-  const NearGeom g = make_geom(h, W, ex, ey);
+size_t direct_scratch_bytes(const ObsDev &h, const NearGeom &g, int slices) {
   const size_t T = (size_t)h.M * h.P;
-  const int p = near_degree(h, g, slices);
-  if (p > 0) return near_sph_scratch_bytes(h, W, ex, ey, p);
+  const int W = g.W;
   size_t b = 0;
   auto add = [&](size_t n) { b += (n + 255) & ~(size_t)255; };
   add(sizeof(double2) * (size_t)W * h.cols * h.P);     // sigma
@@ -483,6 +479,26 @@ size_t near_image_scratch_bytes(const ObsDev &h, int W, double ex, double ey, in
   add(sizeof(unsigned short) * 2 * (size_t)slices * ((NC + 31) / 32 * 32) * g.Sp);     // B digit tiles
   add(sizeof(double2) * (size_t)tb * NC);                          // C block
   return b;
+}
+
+}  // namespace
+
+size_t near_image_scratch_bytes(const ObsDev &h, int W, double ex, double ey, int slices) {
+  const NearGeom g = make_geom(h, W, ex, ey);
+  const int p = near_degree(h, g, slices);
+  return p > 0 ? near_sph_scratch_bytes(h, W, ex, ey, p) : direct_scratch_bytes(h, g, slices);
+}
+
+// The way of a call with that much scratch: the expansions' degree, 0 for the
+// direct sum, -1 where neither fits. A scratch sized for more waves, which may go
+// the other way, holds one of the two.
+int near_image_way(const ObsDev &h, int W, double ex, double ey, int slices, size_t bytes) {
+  const NearGeom g = make_geom(h, W, ex, ey);
+  const int p = slices > 0 ? near_sph_degree(h, ex, ey, slices) : 0;
+  const bool sph = p > 0 && near_sph_scratch_bytes(h, W, ex, ey, p) <= bytes;
+  const bool direct = direct_scratch_bytes(h, g, slices) <= bytes;
+  if (!sph && !direct) return -1;
+  return sph && (!direct || near_degree(h, g, slices) > 0) ? p : 0;
 }
 
 template <int SD>
@@ -528,10 +544,9 @@ static cudaError_t near_split(const ObsDev *d_o, const ObsDev &h, const NearGeom
 }
 
 cudaError_t launch_near_image(const ObsDev *d_o, const ObsDev &h, int W, const double2 *coef,
-                              double ex, double ey, const double *dirs, int slices, double2 *U,
+                              double ex, double ey, const double *dirs, int slices, int p, double2 *U,
                               void *scratch, cudaStream_t st) {
   const int T = h.M * h.P;
-  const int p = near_degree(h, make_geom(h, W, ex, ey), slices);
   if (p > 0) return launch_near_sph(d_o, h, W, coef, ex, ey, dirs, p, U, scratch, st);
   char *sc = static_cast<char *>(scratch);
   double2 *sigma = reinterpret_cast<double2 *>(sc);

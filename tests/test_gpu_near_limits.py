@@ -102,3 +102,23 @@ def test_near_ring_close_to_the_axis(rho):
     c = rng.standard_normal((3, P, N)) + 1j * rng.standard_normal((3, P, N))
     err = _against_direct(op, k, (3.4, 3.4), c, 7)
     assert err < 1.5e-13, err
+
+
+def test_near_scratch_of_more_waves():
+    """A scratch sized for 30 waves (which take the direct sum here) serves every smaller
+    number of waves on the same lattice, whichever way they would go with their own."""
+    from paper_1506_05083_gb300 import axi
+    N, P, k, lat = 24, 18, 2.5, (2.85, 2.85)
+    op = _operator(N, P, k)
+    rng = np.random.default_rng(1)
+    c = torch.tensor(rng.standard_normal((30, P, N)) + 1j * rng.standard_normal((30, P, N)), device="cuda")
+    d = torch.tensor(synth.plane_wave_directions(30, 3), device="cuda")
+    need = axi._near_bytes(op, 0, 30, lat, 7)
+    scratch = torch.empty(need, dtype=torch.uint8, device="cuda")
+    for W in (30, 17, 8, 3, 1):
+        args = (op, c[:W].contiguous(), lat, d[:W].contiguous())
+        U = axi.near_image_sum(*args, slices=7, scratch=scratch)
+        ref = axi.near_image_sum(*args, slices=0)
+        assert (U - ref).abs().max() < 2.0 ** -44 * N * P * ref.abs().max(), W
+    with pytest.raises(axi.AxiError):
+        axi.near_image_sum(*args, slices=7, scratch=scratch[:1 << 16])
