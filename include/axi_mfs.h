@@ -97,7 +97,8 @@ typedef enum {
  * singular values >= 1e-10 sigma_max (the paper's truncation), as two
  * products and a scaling: the pseudo-inverse is never formed. The workspace
  * holds U_R, V and Sigma per mode (2 N^2 + N numbers) and N 32-bit integers.
- * R is preconditioned by a QR with column pivoting (see axi_svd_jacobi). A
+ * R of more than 23 columns is preconditioned by a QR with column pivoting
+ * (see axi_svd_jacobi). A
  * mode whose Jacobi sweeps do not converge in 40 latches AXI_ERR_TIMEOUT. */
 #define AXI_PLAN_TSVD ((int32_t)1 << 17)
 
@@ -416,10 +417,14 @@ axi_status axi_fill_c(const axi_operator *op, int32_t obs, const axi_cell *cell,
  * columns of X = P R1^H, which are graded and nearly orthogonal, and end with
  * X = V Sigma. A sweep orders the columns by decreasing norm (d_sigma holds
  * that order during the call) and rotates every column pair once, by pairs of
- * column blocks that meet in rounds of disjoint pairs; the sweeps stop when
- * every pair's |x^H y| / (||x|| ||y||) is at most tol (e.g. 1e-15), after at
+ * column blocks that meet in rounds of disjoint pairs (single pairs where two
+ * columns of m + n values exceed an SM's shared memory, m + n above about
+ * 7000); the sweeps stop when every pair's |x^H y| / (||x|| ||y||) is at most tol (e.g. 1e-15), after at
  * most max_sweeps. *sweeps receives the number run. The call synchronises
  * `stream` after the QR and after every sweep (not under stream capture).
+ * Singular values of a matrix with scaled columns come out to their own
+ * rounding, empty columns (norms below 2^-505) as exact zeros, which
+ * axi_svd_solve drops at any cutoff.
  * Device buffers are the caller's, 16-byte aligned (8 for d_sigma).
  * Errors: AXI_ERR_ARG, AXI_ERR_NUMERIC (not converged in max_sweeps, or a
  * non-finite value), AXI_ERR_CUDA.
@@ -673,8 +678,10 @@ axi_status axi_eval_field(const axi_operator *op, int32_t obs, int32_t W,
  *             (the lattice's 90-degree symmetry is used when e_x = e_y and 4 | P),
  *             or, where a rule on the sizes expects it to be faster, the same sum
  *             by spherical-wave expansions in FP64 about the obstacle's centre
- *             (the images lie outside the sphere that holds the obstacle), to
- *             about 2e-15 of the sum.
+ *             (the images lie outside the sphere that holds the obstacle), where
+ *             they keep the digits asked for: up to k r = 35 for 7 (r the radius of
+ *             that sphere), 55 for fewer. For the cup (k r = 30) the error is
+ *             1.3e-14 of the sum, 3.1e-14 by 7 digits.
  *   d_out   : device [W][M*P], target index t = m*P + l.
  *   d_scratch, scratch_bytes : >= axi_near_image_workspace_bytes() for this
  *             lattice and slices and for W or more waves; the split path stages

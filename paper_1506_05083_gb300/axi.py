@@ -642,8 +642,8 @@ def periodic_iter_apply(op, g: torch.Tensor, lattice, dirs: torch.Tensor, C_blk:
                         cutoff=1e-10, near_slices=0, obs=0, want_coef=False, out=None, stream=None):
     """One application of eq. iter's operator, y = (I + A_else A_0^+ -
     B Q^+ C A_0^+) g, on Neumann boundary samples g [W][M][P]: the operator's
-    apply, the near-image sum (FP64 direct for near_slices 0, else split into
-    that many digits on tensor cores), C eta, the SVD solve with Q's factors
+    apply, the near-image sum (FP64 direct for near_slices 0, else to that many
+    digits, split on tensor cores or by expansions), C eta, the SVD solve with Q's factors
     (US, V, sigma of `svd_jacobi`) and the combine, each through its own C
     entry point on `stream`. C_blk from `Operator.c_block`, bt from
     `Operator.btilde` (degree p). Returns y [W][M][P] (and A_0^+ g, [W][P][N],

@@ -49,7 +49,7 @@
 
 namespace axi {
 namespace {
-// (cos, sin)(2 pi i / 1024) with 62 fractional bits for trig::sincos_ring_q
+// (cos, sin)(2 pi i / 1024) with 62 fractional bits for trig::sincos_phase
 __device__ const long long g_ring_q62[1024][2] = {
 #include "ring_table_q62.inc"
 };

@@ -8,7 +8,7 @@
 // (the azimuthal sum of a ring's P points against e^{-i m phi} is the ring's
 // coefficient of mode m mod P, so the P-point sum is reproduced with its
 // aliases), and near the centre through regular waves L_lm j_l(k r) Y_lm.
-// Degrees l <= p reach FP64 rounding (sph_degree); p is 72 for the k = 25
+// Degrees l <= p reach FP64 rounding (near_sph_degree); p is 72 for the k = 25
 // cup. The direct sum costs M P N P kernel values per image, in FP64 on a
 // part with 1/64-rate FP64; this one costs O(p^2 (N + M) + p^3) per wave, all
 // of it small real-by-complex matrix products.

@@ -993,9 +993,6 @@ cudaError_t launch_qr_panel(const ObsDev *d_obs, const int *d_task_obs, const in
   return cudaGetLastError();
 }
 
-// The next panel's kNB columns, in native FP64 with narrow tiles (two CTAs
-// per mode): this update is on the critical path of the factorisation, where
-// the split path would first need the panel's digits.
 namespace {
 
 template <typename K, typename... Args>
@@ -1039,6 +1036,10 @@ cudaError_t launch_apply_qh_fp64(const ObsDev *d_o, const ObsDev &h, double2 *X,
 
 }  // namespace
 
+// The next panel's kNB columns in native FP64: this update is on the critical
+// path of the factorisation. Rows over a cluster of 8 or 4 CTAs of 16 rows or
+// more, else of 2, while the clusters fit one wave; beyond that two CTAs a
+// mode, by columns.
 cudaError_t launch_qr_update_next(const ObsDev *d_obs, const int *d_task_obs,
                                   const int *d_task_mode, int ntasks, int p, int rows, cudaStream_t st) {
   if (ntasks <= 0) return cudaSuccess;
@@ -1057,6 +1058,8 @@ cudaError_t launch_qr_update_next(const ObsDev *d_obs, const int *d_task_obs,
   return launch_clusters(qr_next_rows_kernel<kTA, 1>, dim3(ntasks, kNB / kTA), kNB * kTA, 1, st, d_obs, d_task_obs,
                          d_task_mode, p);
 }
+
+// Columns from kNB past the panel onward, native FP64 or split digits.
 cudaError_t launch_qr_update_rest(const ObsDev *d_obs, const int *d_task_obs,
                                   const int *d_task_mode, int ntasks, int p, int slices,
                                   int max_rest_cols, int rest_grid, bool use_y, cudaStream_t st) {
