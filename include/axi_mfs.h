@@ -679,7 +679,7 @@ axi_status axi_eval_field(const axi_operator *op, int32_t obs, int32_t W,
  *             or, where a rule on the sizes expects it to be faster, the same sum
  *             by spherical-wave expansions in FP64 about the obstacle's centre
  *             (the images lie outside the sphere that holds the obstacle), where
- *             they keep the digits asked for: up to k r = 35 for 7 (r the radius of
+ *             they keep the digits asked for: up to k r = 45 for 7 (r the radius of
  *             that sphere), 55 for fewer. For the cup (k r = 30) the error is
  *             1.3e-14 of the sum, 3.1e-14 by 7 digits.
  *   d_out   : device [W][M*P], target index t = m*P + l.

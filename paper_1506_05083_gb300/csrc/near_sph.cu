@@ -51,8 +51,8 @@
 // 1e-12 for 60 (k r is that of the larger radius). Measured, single sources at 1.3
 // (r_s + r_t), against the direct sum of 7 digits: 6e-15 and 7e-15 for k r = 20, 1.7e-14
 // and 1.0e-14 for 33, 2.0e-14 and 1.6e-14 for 45, 1.6e-13 and 1.7e-14 for 57; 6 digits
-// keep 5e-13. So a caller who asks for 7 digits takes this path up to k r = 35,
-// with fewer up to 55 (near_sph_degree). T depends on |m|, and
+// keep 5e-13. So a caller who asks for 7 digits (2^-44 = 6e-14) takes this path up to
+// k r = 45, with fewer up to 55 (near_sph_degree). T depends on |m|, and
 // M'_{-m}(-c) = (-1)^l M'_m(c), so the sums over even and odd l' give (m, c)
 // and (-m, -c) together.
 #include <algorithm>
@@ -885,7 +885,7 @@ int near_sph_degree(const ObsDev &h, double ex, double ey, int slices) {
   const double D = std::min(ex, ey), rs = h.sph_rs, rt = h.sph_rt;
   if (!(rs > 0.0) || !(rt > 0.0) || !(h.sph_rho_min > 1e-6 * rt) || !(D > 1.02 * (rs + rt))) return 0;
   const double r = std::max(rs, rt);
-  if (!(h.k * r <= (slices >= 7 ? 35.0 : 55.0)) || !(h.k * std::hypot(ex, ey) < 0x1p19) || !(h.k * (D - r) > 0x1p-100)) return 0;
+  if (!(h.k * r <= (slices >= 7 ? 45.0 : 55.0)) || !(h.k * std::hypot(ex, ey) < 0x1p19) || !(h.k * (D - r) > 0x1p-100)) return 0;
   constexpr int L = 2 * kSphMaxDegree + 2;
   int ja[L + 1], jb[L + 1], ha[L + 1], hb[L + 1];
   constexpr int L1 = kSphMaxDegree + 1;

@@ -60,7 +60,7 @@ def test_near_far_lattices(lat):
     assert err < 1.5e-13 + 4 * 2.0 ** -53 * k * np.hypot(*lat), err
 
 
-@pytest.mark.parametrize("kr,slices", [(34.0, 7), (57.0, 7), (54.0, 6), (60.0, 6), (34.0, 4)])
+@pytest.mark.parametrize("kr,slices", [(34.0, 7), (44.5, 7), (57.0, 7), (54.0, 6), (60.0, 6), (34.0, 4)])
 def test_near_large_kr(kr, slices):
     """One source a wave, so that the error is relative to single kernel values: a
     split call keeps the digits it was asked for, 2^(-7 slices + 5), whether the
